@@ -227,14 +227,13 @@ int df_set_tile_shapes(df_ctx* ctx, const int* shapes);
 /* Transport kernels (Sec. 3.1 sweeps).  DF_TRANSPORT_SEPARATE: four kernels per sweep
  * (e/rho and Pi/rho_face; mass and energy fluxes; momentum fluxes; conservative
  * update) exchanging their results through HBM.  DF_TRANSPORT_FUSED: one kernel per
- * sweep that keeps them in shared memory for a tile plus its halo (the halo's
- * quotients and fluxes are recomputed by neighbouring tiles) and ping-pongs the
- * state through a second copy; about a third of the memory traffic.  The two give
- * the same arithmetic on every active cell (equal up to the compiler's contraction
- * of multiply-adds).  DF_TRANSPORT_AUTO (default): separate for DF_FP64 (its
- * kernels are bound by the FP64 pipe); for DF_FP32_STATE fused in pools of several
- * runs and, for a single run, on levels of at least 512 Ki active cells (the sweeps
- * leave one small box short of blocks). */
+ * sweep that keeps them in registers while each warp marches through the box, and
+ * passes the state from sweep to sweep through scratch planes; about a third of the
+ * memory traffic.  The two give the same arithmetic on every active cell up to rounding
+ * (the compiler's contraction of multiply-adds; at the x sweep the fused form forms the
+ * momenta from v and rho; in double-float it leaves more intermediate sums
+ * unnormalised).  DF_TRANSPORT_AUTO (default): separate for DF_FP64, fused for
+ * DF_FP32_STATE. */
 #define DF_TRANSPORT_AUTO 0
 #define DF_TRANSPORT_SEPARATE 1
 #define DF_TRANSPORT_FUSED 2

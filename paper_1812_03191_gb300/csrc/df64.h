@@ -114,6 +114,25 @@ __host__ __device__ __forceinline__ df64 div_u(df64 a, df64 b) {
   return df64(q1, rem * r);
 }
 
+// A sum and a difference without the final renormalisation, for results that only feed
+// products, quotients and further sums: the value and its error are the operators', but
+// after a cancellation lo may be as large as hi.  It stays below 2^-23 (|a| + |b|), so
+// what a product or quotient drops of it (lo times the other operand's lo) is below
+// 2^-46 of |a| + |b| times that operand: the size of the sum's own error.  Not for sign
+// tests, canonical(), to_double() or an ordered comparison.
+__host__ __device__ __forceinline__ df64 add_u(df64 a, df64 b) {
+  const df64 s = two_sum(a.hi, b.hi);
+  return df64(s.hi, s.lo + (a.lo + b.lo));
+}
+__host__ __device__ __forceinline__ df64 sub_u(df64 a, df64 b) { return add_u(a, -b); }
+// p - a for a float p, likewise
+__host__ __device__ __forceinline__ df64 fsub_u(float p, df64 a) {
+  const df64 s = two_sum(p, -a.hi);
+  return df64(s.hi, s.lo - a.lo);
+}
+// any pair as a normalised one
+__host__ __device__ __forceinline__ df64 norm(df64 a) { return two_sum(a.hi, a.lo); }
+
 __host__ __device__ __forceinline__ df64 scale(df64 a, float p2) {
   return df64(a.hi * p2, a.lo * p2);
 }

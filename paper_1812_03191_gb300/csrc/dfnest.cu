@@ -362,9 +362,6 @@ int run_create(Run** out, int n_levels, const int n0[3], const int n[3], const d
     r->S.F = b + plane * 7;
     r->S.E = b + plane * 8;
     for (int m = 0; m < 3; ++m) r->S.P[m] = b + plane * (9 + m);
-    r->S.qb[0] = r->S.eps;
-    for (int m = 0; m < 3; ++m) r->S.qb[1 + m] = r->S.w[m];
-    r->S.qb[4] = r->S.P[0];
   }
   CKR(dev_alloc(r->al, (void**)&r->ds, sizeof(DevScalars)));
   CKR(cudaMemset(r->ds, 0, sizeof(DevScalars)));
@@ -558,21 +555,13 @@ struct TileTable {
   }
 };
 
-// Transport of one level step: DF_TRANSPORT_FUSED or DF_TRANSPORT_SEPARATE as set.
-// DF_TRANSPORT_AUTO picks separate kernels for FP64, whose kernels are bound by the
-// FP64 pipe, which the halo arithmetic the sweeps repeat would load further.  For
-// the FP32 state it picks fused sweeps in pools, whose merged launches give the
-// sweeps blocks enough (and a run must get the same bits whatever it shares its
-// pool with), and for a context's levels of at least kFusedMinCells active cells.
-// A fused sweep's blocks march through whole columns, so one small box leaves the
-// GPU short of blocks: on GB300 the separate kernels win for one run of 3 x 64^3
-// levels, the sweeps from 3 x 96^3, and the sweeps win for pools of small runs.
-constexpr long long kFusedMinCells = 512 * 1024;
-
-bool sweeps_fused(int mode, int prec, const LevelView& v, bool pool) {
+// Transport of one level step: DF_TRANSPORT_FUSED or DF_TRANSPORT_SEPARATE as set;
+// DF_TRANSPORT_AUTO takes the fused sweeps for the FP32 state (against the separate
+// kernels, per coarse step: 3 x 64^3 0.47 to 0.59 ms, nine quadrant levels of 32x32x64
+// 27.8 to 32.1) and the separate kernels for FP64 (nine quadrant levels 41.4 to 44.4).
+bool sweeps_fused(int mode, int prec) {
   if (mode != DF_TRANSPORT_AUTO) return mode == DF_TRANSPORT_FUSED;
-  return prec == DF_FP32_STATE &&
-         (pool || (long long)v.n[0] * v.n[1] * v.n[2] >= kFusedMinCells);
+  return prec == DF_FP32_STATE;
 }
 
 template <class T>
@@ -587,6 +576,8 @@ struct Builder {
   TileTable tiles;
   int transport = DF_TRANSPORT_AUTO;  // per level: fused sweeps or separate kernels
   bool pool = false;                  // the plan steps a pool (else a context)
+  int sm_count = 148;                 // SMs of the device
+  long long pool_cells = 0;           // a pool's finest levels: their active cells
   mutable unsigned br = 0;  // second sub-cycles enclosing the items being added
   mutable int sub_of[DF_MAX_LEVELS] = {};  // sub-cycle of each level being added
 
@@ -629,22 +620,26 @@ struct Builder {
     return it;
   }
 
-  // planes per chunk of a fused sweep's marching axis, at least 8 (16 when marching
-  // along the sweep, whose chunks start 3 planes early and finish 2 planes late).
-  // A context's sweep launches one block per (column, chunk): as many chunks as
-  // leave every block resident at once (one wave: the SMs times the blocks of that
-  // kernel an SM holds, when that is at least two), since each chunk repeats the
-  // planes of its halo.  A pool's persistent blocks take chunks in turn: about 600
-  // chunks balance them.
+  // Planes per chunk of a fused sweep over box b.  A context: as many chunks as leave
+  // every block resident at once, but at least 4 planes (x sweep: 1) each, since a chunk
+  // repeats 5 (1) (levels of 32^3 to 64^3: 6 planes ran up to 8 % slower per coarse
+  // step, 1 to 3 planes no faster).  A pool: its launches hold every run's sweep, so the
+  // chunk is what gives about 2000 blocks in all, within 8 and 32 planes (24 runs of 32^3
+  // to 96^3: 8.06 ms a step with 6 planes, 7.26 with 24, 7.40 with 40; 16 runs of 24^3 to
+  // 32^3: 0.99 with 12, 1.17 with 24).
   int sweep_chunk(const Box& b, int d) const {
-    const int ra = sweep_row_axis(d), mu = sweep_march_axis(d), ow = sweep_own_x(d);
-    const int ncols = ((b.hi[0] - b.lo[0] + ow - 1) / ow) *
-                      ((b.hi[ra] - b.lo[ra] + kSweepRows - 1) / kSweepRows);
-    const int nm = b.hi[mu] - b.lo[mu];
-    const int slots = pool ? 600 : sweep_slots((int)sizeof(T), d);
-    const int chunks = std::max(1, slots / std::max(1, ncols));
-    const int zc = (nm + chunks - 1) / chunks;
-    return std::min(nm, std::max(zc, d == 0 ? 8 : 16));
+    const int mu = sweep_march_axis(d), nm = b.hi[mu] - b.lo[mu];
+    int zc;
+    if (pool) {
+      const long long fit = pool_cells / (sweep_own(1) * (kSweepThreads / 32)) / 2000;
+      zc = (int)std::min<long long>(std::max<long long>(fit, 8), 32);
+      if (d == 0) zc /= 2;
+    } else {
+      const int slots = sm_count * sweep_blocks((int)sizeof(T), d);
+      const int chunks = std::max(1, slots / std::max(1, sweep_columns(b, d)));
+      zc = std::max((nm + chunks - 1) / chunks, d == 0 ? 1 : 4);
+    }
+    return std::min(nm, zc);
   }
 
   // margin boxes (active cells +- margin) unless verifying with whole arrays or the
@@ -670,7 +665,7 @@ struct Builder {
 
   void add(std::vector<Entry>& out, int op, int d, Item<T> it) const {
     it.b.tile = is_box_op(op) ? tiles.t[op][d] : 0;
-    it.b.zc = op == OP_SWEEP ? sweep_chunk(it.b, d) : 0;
+    if (op == OP_SWEEP) it.b.zc = sweep_chunk(it.b, d);
     it.br = br;
     it.count = op_count(op, d, it.L, it.F, it.b);
     out.push_back({op, d, it});
@@ -689,6 +684,10 @@ struct Builder {
 
   void level_step(const Run& r, int l, int m_out, std::vector<Entry>& out) const {
     Item<T> it = base(r, l);
+    const bool fused_tr =
+        sweeps_fused(transport, sizeof(T) == 8 ? DF_FP64 : DF_FP32_STATE);
+    // the x sweep forms the staggered momenta from v and rho itself
+    if (fused_tr) it.flags &= ~FL_WRITE_PI;
     it.b = box(it.L, m_out + kReach, r.P.av_c2 > 0.0, l == 0 ? 1 : 0);
     const Phys& P = r.P;
     // The two sub-cycles of a finest level follow each other with nothing in between
@@ -714,8 +713,6 @@ struct Builder {
       add(out, OP_VISC_V, 0, it);
     }
     if (P.hydro_on || P.L != 0.0 || P.chi > 0.0) add(out, OP_COMPRESS, 0, it);
-    const bool fused_tr =
-        sweeps_fused(transport, sizeof(T) == 8 ? DF_FP64 : DF_FP32_STATE, it.L, pool);
     // before the separate transport kernels the diffusion also forms the x sweep's
     // e/rho (in Scratch::w[0]), in place of that sweep's preparation kernel
     const bool eps_x = P.chi > 0.0 && P.hydro_on && !fused_tr;
@@ -724,12 +721,8 @@ struct Builder {
       add(out, OP_DIFFUSE, eps_x ? 1 : 0, it);
     }
     if (P.hydro_on && fused_tr) {
-      for (int d = 0; d < 3; ++d) {
-        add(out, OP_SWEEP, d, it);
-      }
-      Item<T> vr = it;
-      vr.flags |= FL_FUSED;
-      add(out, OP_VREC, vrec_d, vr);
+      for (int d = 0; d < 3; ++d) add(out, OP_SWEEP, d, it);
+      add(out, OP_VREC, vrec_d, it);
     } else if (P.hydro_on) {
       // At the x sweep the staggered momenta were just formed from v and rho (the
       // kick, or the viscosity stage after it, wrote them; nothing since has changed
@@ -885,7 +878,7 @@ int plan_upload(Plan& plan) {
 
 template <class T>
 int plan_build(Plan& plan, const std::vector<Run*>& runs, int full_boxes,
-               const TileTable& tiles, int transport, bool pool) {
+               const TileTable& tiles, int transport, bool pool, int sm_count) {
   plan_invalidate(plan);
   plan.prec = sizeof(T) == 8 ? DF_FP64 : DF_FP32_STATE;
   size_t nr = runs.size();
@@ -901,6 +894,11 @@ int plan_build(Plan& plan, const std::vector<Run*>& runs, int full_boxes,
   B.tiles = tiles;
   B.transport = transport;
   B.pool = pool;
+  B.sm_count = sm_count;
+  for (const Run* r : runs) {
+    const LevelView& v = r->L[r->nl - 1].v;
+    B.pool_cells += (long long)v.n[0] * v.n[1] * v.n[2];
+  }
   B.per_run.resize(nr);
   for (size_t r = 0; r < nr; ++r) B.coarse_step(*runs[r], (int)r, B.per_run[r]);
   B.merge(plan);
@@ -1192,9 +1190,10 @@ int sync_health(cudaStream_t st, Run* r) {
 }
 
 int build_plan(Plan& p, const std::vector<Run*>& runs, int prec, int full_boxes,
-               const TileTable& tiles, int transport, bool pool) {
-  return prec == DF_FP64 ? plan_build<double>(p, runs, full_boxes, tiles, transport, pool)
-                         : plan_build<float>(p, runs, full_boxes, tiles, transport, pool);
+               const TileTable& tiles, int transport, bool pool, int sm_count) {
+  return prec == DF_FP64
+             ? plan_build<double>(p, runs, full_boxes, tiles, transport, pool, sm_count)
+             : plan_build<float>(p, runs, full_boxes, tiles, transport, pool, sm_count);
 }
 
 // state of the runs that tuning steps disturb (fields, scalars, force-ring cursor)
@@ -1309,7 +1308,7 @@ int autotune(const std::vector<Run*>& runs, Exec& x, int prec, int transport, Ti
       for (int d = 0; d < 3; ++d) tt.t[o][d] = tk;
     Plan p;
     p.al = runs.empty() ? Allocator() : runs[0]->al;
-    rc = build_plan(p, runs, prec, 0, tt, transport, !single_fast);
+    rc = build_plan(p, runs, prec, 0, tt, transport, !single_fast, x.sm_count);
     if (!rc) rc = time_plan(p, x, prec, 0, single_fast, per);
     plan_free(p);
     for (int o = 0; o < OP_COUNT && !rc; ++o)
@@ -1330,7 +1329,7 @@ int autotune(const std::vector<Run*>& runs, Exec& x, int prec, int transport, Ti
     }
     Plan p;
     p.al = runs.empty() ? Allocator() : runs[0]->al;
-    rc = build_plan(p, runs, prec, 0, tiles, transport, !single_fast);
+    rc = build_plan(p, runs, prec, 0, tiles, transport, !single_fast, x.sm_count);
     for (int gi = 0; gi < 6 && !rc; ++gi) {
       rc = time_plan(p, x, prec, cand[gi], single_fast, per);
       for (int o = 0; o < OP_COUNT && !rc; ++o) {
@@ -1477,7 +1476,8 @@ int df_step(df_ctx* c, int n, double* t_out) {
   // the search drops second sub-cycles on the device), replayed from a graph
   for (int l = 0; l < r->nl; ++l) r->xi[l] = 2;
   if (!c->plan.valid)
-    rc = build_plan(c->plan, runs, r->prec, c->full_boxes, c->tiles, c->transport, false);
+    rc = build_plan(c->plan, runs, r->prec, c->full_boxes, c->tiles, c->transport, false,
+                    c->x.sm_count);
   if (!rc) rc = step_plan(c->plan, c->x, r->prec, n);
   leave(c);
   r->stepped = true;
@@ -1955,7 +1955,8 @@ int df_pool_step(df_pool* p, int n) {
   if (runs.empty() || n == 0) return DF_OK;
   DevGuard g(p->device);
   int rc = DF_OK;
-  if (!p->plan.valid) rc = build_plan(p->plan, runs, p->prec, 0, p->tiles, p->transport, true);
+  if (!p->plan.valid)
+    rc = build_plan(p->plan, runs, p->prec, 0, p->tiles, p->transport, true, p->x.sm_count);
   if (rc) return rc;
   enter(p);
   rc = step_plan(p->plan, p->x, p->prec, n);

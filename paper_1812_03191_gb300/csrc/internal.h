@@ -53,9 +53,6 @@ struct Scratch {
   void* F;      // mass flux of the current sweep
   void* E;      // energy flux of the current sweep
   void* P[3];   // momentum fluxes of the current sweep
-  // second copy of (rho, e, Pi_x, Pi_y, Pi_z) for the fused sweeps (planes of eps,
-  // w and P[0], which the fused path does not use): x writes it, y reads it, z writes it
-  void* qb[5];
 };
 
 // Box of a stencil op.  tile = 0: elements enumerated x fastest over the box;
@@ -101,20 +98,54 @@ __host__ __device__ inline int tile_extent(int k, int axis) {
   }
 }
 
-// Fused transport sweep: a block of kSweepRows + 1 warps; each warp holds one row
-// of 32 consecutive x positions (a few of them halo for the x-stencil), the extra
-// warp the row below the block's rows, and the block marches through zc planes of
-// the marching axis (z for the x sweep, the sweep axis itself for y and z).
-constexpr int kSweepRows = 8;
-constexpr int kSweepThreads = 32 * (kSweepRows + 1);
-__host__ __device__ inline int sweep_own_x(int d) { return d == 0 ? 27 : 31; }
+// Fused transport sweep (el_sweep, kernels.cu).  Blocks of 4 warps; smaller and larger
+// ones measured the same.  Blocks an SM is to hold set the registers: 128 (y, z) and 80
+// (x) for FP32, 168 and 128 in double-float, the most that does not spill much; one block
+// more or fewer ran 2-30 % slower.
+constexpr int kSweepThreads = 128;
+__host__ __device__ constexpr int sweep_blocks(int esz, int d) {
+  return esz == 8 ? (d == 0 ? 4 : 3) : (d == 0 ? 6 : 4);
+}
 __host__ __device__ inline int sweep_row_axis(int d) { return d == 1 ? 2 : 1; }
 __host__ __device__ inline int sweep_march_axis(int d) { return d == 0 ? 2 : d; }
+// double-float: planes of the march in flight, and the arrays of a plane
+constexpr int kSweepStages = 3;
+constexpr int kSweepArrays = 8;
+// values of the buffer of the planes in flight (FP32 keeps its one plane in registers)
+__host__ __device__ constexpr int sweep_ahead(int esz) {
+  return esz == 8 ? kSweepStages * kSweepArrays * kSweepThreads : kSweepThreads;
+}
+// positions a warp owns, and halo positions of a row
+__host__ __device__ constexpr int sweep_own(int d) { return d == 0 ? 27 : 31; }
+__host__ __device__ constexpr int sweep_halo(int d) { return d == 0 ? 5 : 1; }
+// blocks that cover the rows of box b side by side; units: times the chunks of the march
+__host__ __device__ inline int sweep_columns(const Box& b, int d) {
+  const int ra = sweep_row_axis(d), n = sweep_own(d) * (kSweepThreads / 32);
+  return ((b.hi[0] - b.lo[0] + sweep_halo(d)) * (b.hi[ra] - b.lo[ra]) + n - 1) / n;
+}
+// Position of lane `lane` of the w-th warp along those rows; false past their end.  A
+// warp owns sweep_own consecutive positions and repeats its neighbours' as halo; `mine`:
+// an owned position (of the box or of a row's halo).  Past either end of the rows a lane
+// repeats the last position, so that it always reads inside the box and its halo.
+struct SweepLane {
+  int x, row;
+  bool mine;
+};
+__host__ __device__ inline bool sweep_lane(const Box& b, int d, int w, int lane, SweepLane& p) {
+  const int lo = d == 0 ? 3 : 1, own = sweep_own(d), ra = sweep_row_axis(d);
+  const int pitch = b.hi[0] - b.lo[0] + sweep_halo(d);
+  const int len = pitch * (b.hi[ra] - b.lo[ra]);
+  if (w * own >= len) return false;
+  const int f = w * own - lo + lane;
+  const int c = f < 0 ? 0 : f < len ? f : len - 1, r = c / pitch;
+  p.x = b.lo[0] - lo + c - r * pitch;
+  p.row = b.lo[ra] + r;
+  p.mine = lane >= lo && lane < lo + own && f < len;
+  return true;
+}
 __host__ __device__ inline int sweep_units(const Box& b, int d) {
-  const int ra = sweep_row_axis(d), mu = sweep_march_axis(d), ow = sweep_own_x(d);
-  const int nsx = (b.hi[0] - b.lo[0] + ow - 1) / ow;
-  const int nsr = (b.hi[ra] - b.lo[ra] + kSweepRows - 1) / kSweepRows;
-  return nsx * nsr * ((b.hi[mu] - b.lo[mu] + b.zc - 1) / b.zc);
+  const int mu = sweep_march_axis(d);
+  return sweep_columns(b, d) * ((b.hi[mu] - b.lo[mu] + b.zc - 1) / b.zc);
 }
 
 struct Phys {
@@ -333,7 +364,6 @@ __host__ __device__ inline long long cu_chunks(const int* n, int G) {
 
 enum ItemFlags {
   FL_WRITE_PI = 1, FL_SS3 = 2, FL_LUM = 4, FL_EPS = 8, FL_DFR = 16, FL_HYDRO = 32,
-  FL_FUSED = 64,  // VREC: the transport ran as fused sweeps (state in Scratch::qb)
   FL_EPS_ONLY = 128  // TPREP: e/rho only (the x sweep reads Pi/rho_face - V from v)
 };
 
@@ -389,7 +419,6 @@ template <class T>
 int launch_batch(int op, int d, const Item<T>* items, const unsigned* starts, int nitems,
                  unsigned nchunks, unsigned grid, cudaStream_t st, const Item<T>* host_item);
 int op_chunk_elems(int op, int esz);  // elements per chunk for state elements of esz bytes
-int sweep_slots(int esz, int d);      // a context's sweep blocks resident at once
 unsigned op_count(int op, int d, const LevelView& L, const LevelView& F, const Box& b);
 int force_partials_per_level(const LevelView& L);
 int launch_force_weights(const LevelView& L, const Phys& P, cudaStream_t st);

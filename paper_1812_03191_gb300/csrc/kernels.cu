@@ -81,6 +81,11 @@ __device__ __forceinline__ df64 hdiv(df64 a, df64 b) { return a / b; }
 // without the final renormalisation (mul_u, div_u in df64.h), in FP32 the plain ones
 __device__ __forceinline__ float mul_u(float a, float b) { return a * b; }
 __device__ __forceinline__ float div_u(float a, float b) { return __fdividef(a, b); }
+// likewise the sum, the difference and p - a of a float p (add_u, sub_u, fsub_u there)
+__device__ __forceinline__ float add_u(float a, float b) { return a + b; }
+__device__ __forceinline__ float sub_u(float a, float b) { return a - b; }
+__device__ __forceinline__ float fsub_u(float p, float a) { return p - a; }
+__device__ __forceinline__ float norm(float a) { return a; }
 
 // The stencils' arithmetic type C = Arith<T> (internal.h): float for the FP32 state,
 // double-float for the FP64 state.  Loads convert the stored value to C, stores round
@@ -121,7 +126,7 @@ __device__ __forceinline__ df64 ky_add(df64 k, df64 y, df64 z) {
 // consumers only take differences of it, so the quotient stays unnormalised.
 template <class C, class B>
 __device__ __forceinline__ C eps_dev(C de, C dr, const B& bg) {
-  return div_u(de - mul_u(bg.eps0, dr), bg.rho0 + dr);
+  return div_u(sub_u(de, mul_u(bg.eps0, dr)), add_u(bg.rho0, dr));
 }
 // a value as a store of the state keeps it (the FP64 state's stores cut lo)
 __device__ __forceinline__ float as_stored(float v) { return v; }
@@ -175,7 +180,7 @@ __device__ __forceinline__ bool lt0(float v) { return v < 0.f; }
 template <class C>
 __device__ __forceinline__ C hslope(C dl, C dr) {
   C pr = mul_u(dl, dr);
-  return le0(pr) ? C(0.f) : div_u(pr, dl + dr);
+  return le0(pr) ? C(0.f) : div_u(pr, add_u(dl, dr));
 }
 
 // The upwind side's value, slopes and coefficient are selected first, so one limiter
@@ -198,7 +203,7 @@ __device__ __forceinline__ C upwind_v(C qmm, C qm, C q0, C qp, C u, C cour) {
     dl = a - (up ? qmm : qm);
     dr = (up ? q0 : qp) - a;
   }
-  return a + mul_u((up ? C(1.f) : C(-1.f)) - cour, hslope(dl, dr));
+  return add_u(a, mul_u(fsub_u(up ? 1.f : -1.f, cour), hslope(dl, dr)));
 }
 
 template <class P, class C>
@@ -786,37 +791,6 @@ __device__ __forceinline__ void el_tupdate(const LevelView& L, const Box& b, con
   }
 }
 
-// ------------------------------------------------------- fused transport sweep
-// One sweep along d (Sec. 3.1 transport: the mass flux F = rho* v A dt with the
-// time-centred van Leer value rho*, e and the momenta carried as (q/rho)* F) with
-// the arithmetic of tprep + tflux + tmom + tupdate, fused and register-blocked.
-// A block is kSweepRows + 1 warps; warp w holds row row0 - 1 + w (the first is the
-// halo row below the block's rows), lane l the x position x0 - hx + l, and the block
-// marches through a chunk of planes of the marching axis.  Values along the marching
-// axis stay in per-thread registers, x neighbours come by warp shuffle, the row
-// below through one shared-memory exchange per plane.
-//   y, z sweeps: march along the sweep; the stencil along d is the register window.
-//   x sweep: march along z; the stencil along x is a shuffle (3 halo lanes below,
-//            2 above), the z neighbour is the previous plane's registers.
-// Ping-pong state: the sweep reads `src` inside the box and the level's own arrays
-// outside it (the values the separate kernels, which update in place, read there)
-// and writes every box cell it owns to `dst`: x and z sweeps from the level's
-// arrays to Scratch::qb, the y sweep back.  For a child level the fluxes through
-// its frontier faces also go to Scratch::F/E (frontier capture).
-
-__device__ __forceinline__ float shfl_up(float v, int k) {
-  return __shfl_up_sync(0xffffffffu, v, k);
-}
-__device__ __forceinline__ float shfl_dn(float v, int k) {
-  return __shfl_down_sync(0xffffffffu, v, k);
-}
-__device__ __forceinline__ df64 shfl_up(df64 v, int k) {
-  return df64(__shfl_up_sync(0xffffffffu, v.hi, k), __shfl_up_sync(0xffffffffu, v.lo, k));
-}
-__device__ __forceinline__ df64 shfl_dn(df64 v, int k) {
-  return df64(__shfl_down_sync(0xffffffffu, v.hi, k), __shfl_down_sync(0xffffffffu, v.lo, k));
-}
-
 // coarse-level frontier substitution of the low/high d-face fluxes of cell (g); the
 // frontier faces lie on two d-planes, tested first
 template <class C>
@@ -837,337 +811,443 @@ __device__ __forceinline__ void frontier_fluxes(const LevelView& L, int d, const
   }
 }
 
-template <class T, int d>
-__device__ __forceinline__ void el_sweep(const Item<T>& it, unsigned unit,
-                                         Arith<T>* __restrict__ xch) {
+// ------------------------------------------------------- fused transport sweep
+// One sweep along d (Sec. 3.1 transport: the mass flux F = rho* v A dt with the
+// time-centred van Leer value rho*, e and the momenta carried as (q/rho)* F) with
+// the arithmetic of tprep + tflux + tmom + tupdate in one kernel.  Every warp works by
+// itself, without a barrier: a lane holds one position of one row and marches through a
+// chunk of planes.
+//   y, z sweeps (sweep_march): the march is along the sweep; the stencils' values are
+// windows in registers, a chunk starts 3 planes early and ends 2 late.
+//   x sweep (sweep_x): the march is along z; the stencils' values come by warp shuffle, a
+// chunk starts one plane early (mass flux only).
+//   The rows are laid end to end, each with its halo (1 position below; x sweep: 3 below,
+// 2 above), and cut into warps that share 1 (5) positions, so that 96 % (81 %) of the
+// lanes own a cell whatever the box's width; a grid of 32-wide tiles left 80-85 %
+// (71-80 %).  The neighbour below in x comes by shuffle; of the row below the mass flux
+// is formed again from its rho and v_d (a tenth of the arithmetic), which costs less than
+// an exchange between warps: a tile in shared memory with three barriers a plane measured
+// 50 us against 37 at 136^3 (FP32, y), with the same arithmetic per cell.
+//   Each upwind value takes its one-sided differences from a window (x: from the
+// neighbouring lanes), one subtraction per cell and quantity instead of two.
+//   State: x reads the level's rho, e and velocities (at its start the staggered momenta
+// are those of v and rho, so Pi/rho_face - V is the velocity deviation itself and the
+// momenta are formed here), writes Scratch::F, E (rho, e) and Scratch::pi; y reads those
+// and writes Scratch::P[0], P[1] and Scratch::w; z reads those and writes the level's
+// rho and e and Scratch::pi.  Elements outside a box hold what an earlier op left there;
+// no element that is needed later depends on them.
+//   EDGE: the box reaches the ends of the array, where the stencils do not fit (faces 0,
+// 1 and the last along d, face 0 of the other axes).
+//   Bound by instruction issue.  Measured at a 136^3 box (ncu, GB300): FP32 state x 40.5,
+// y 36.9, z 36.8 us, 352 / 314 / 313 lane instructions per cell, against 54-63 us for the
+// earlier form (blocks of 9 warps, one barrier a plane, 363-400 instructions);
+// double-float 137 / 119 / 117 us, 1330 / 1163 / 1162 instructions.
+__device__ __forceinline__ float shfl_up(float v, int k) {
+  return __shfl_up_sync(0xffffffffu, v, k);
+}
+__device__ __forceinline__ float shfl_dn(float v, int k) {
+  return __shfl_down_sync(0xffffffffu, v, k);
+}
+__device__ __forceinline__ df64 shfl_up(df64 v, int k) {
+  return df64(__shfl_up_sync(0xffffffffu, v.hi, k), __shfl_up_sync(0xffffffffu, v.lo, k));
+}
+__device__ __forceinline__ df64 shfl_dn(df64 v, int k) {
+  return df64(__shfl_down_sync(0xffffffffu, v.hi, k), __shfl_down_sync(0xffffffffu, v.lo, k));
+}
+
+// the upwind value (upwind_v) from the two sides' values and the differences
+// dm = q(-1) - q(-2), dc = q(0) - q(-1), dp = q(1) - q(0)
+template <class C>
+__device__ __forceinline__ C upwind_d(C qm, C q0, C dm, C dc, C dp, C u, C cour) {
+  const bool up = gt0(u);
+  return add_u(up ? qm : q0, mul_u(fsub_u(up ? 1.f : -1.f, cour),
+                                   hslope(up ? dm : dc, up ? dc : dp)));
+}
+
+// element access by byte offset from a base that is the same for the whole warp (offsets
+// stay below 2^32: fewer than 2^31 / 5 elements of 8 bytes)
+template <class P>
+__device__ __forceinline__ auto ldb(const P* base, unsigned o) {
+  return ld((const P*)((const char*)base + o), 0);
+}
+template <class P, class C>
+__device__ __forceinline__ void stb(P* base, unsigned o, C v) {
+  st((P*)((char*)base + o), 0, v);
+}
+
+// The planes to come, fetched ahead.  FP32: one plane, in registers (copies into shared
+// memory measured the same).  Double-float: kSweepStages planes by asynchronous copies
+// into shared memory, each thread's values in its own column of the buffer (so no
+// barrier): registers for them would cost a block per SM (y, z: 132 -> 118 us at 136^3,
+// with the unnormalised sums).
+template <class C>
+struct Ahead {
+  static constexpr int NS = 2;
+  C v[kSweepArrays];
+  __device__ __forceinline__ explicit Ahead(C*) {}
+  template <class P>
+  __device__ __forceinline__ void fetch(int a, const P* base, unsigned o) {
+    v[a] = ldb(base, o);
+  }
+  __device__ __forceinline__ void commit() {}
+  __device__ __forceinline__ void take(C (&q)[kSweepArrays]) {
+#pragma unroll
+    for (int a = 0; a < kSweepArrays; ++a) q[a] = v[a];
+  }
+};
+template <>
+struct Ahead<df64> {
+  static constexpr int NT = kSweepThreads, NS = kSweepStages;
+  df64* buf;  // [stage][array][thread], at this thread
+  int in = 0, out = 0;
+  __device__ __forceinline__ explicit Ahead(df64* b) : buf(b) {}
+  template <class P>
+  __device__ __forceinline__ void fetch(int a, const P* base, unsigned o) {
+    const unsigned s = (unsigned)__cvta_generic_to_shared(buf + (in * kSweepArrays + a) * NT);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(s), "l"((const char*)base + o)
+                 : "memory");
+  }
+  __device__ __forceinline__ void commit() {
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    in = in + 1 == NS ? 0 : in + 1;
+  }
+  // the oldest plane in flight, once it has arrived
+  __device__ __forceinline__ void take(df64 (&q)[kSweepArrays]) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(NS - 1) : "memory");
+#pragma unroll
+    for (int a = 0; a < kSweepArrays; ++a) q[a] = buf[(out * kSweepArrays + a) * NT];
+    out = out + 1 == NS ? 0 : out + 1;
+  }
+};
+
+template <class T, int d, bool EDGE>
+__device__ __forceinline__ void sweep_march(const Item<T>& it, int x, int row, bool own, int m0,
+                                            int m1, Arith<T>* __restrict__ buf) {
   using C = Arith<T>;
   constexpr int RA = d == 1 ? 2 : 1;  // row axis
-  constexpr int MU = d == 0 ? 2 : d;  // marching axis
-  constexpr int HX = d == 0 ? 3 : 1;  // halo lanes below the owned x range
-  constexpr int OWNX = d == 0 ? 27 : 31;
-  constexpr int NT = kSweepThreads;
-  constexpr bool kFromB = d == 1;  // x: A -> B, y: B -> A, z: A -> B
+  constexpr unsigned ES = sizeof(C);
   const LevelView& L = it.L;
-  const Box& b = it.b;
-  const Scratch& S = it.S;
-  const Bg<C>& bg = it.bg;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int nsx = (b.hi[0] - b.lo[0] + OWNX - 1) / OWNX;
-  const int nsr = (b.hi[RA] - b.lo[RA] + kSweepRows - 1) / kSweepRows;
-  const int cm = (int)unit / (nsx * nsr), crem = (int)unit - cm * nsx * nsr;
-  const int sr = crem / nsx, sx = crem - sr * nsx;
-  const int x = b.lo[0] + sx * OWNX - HX + lane;
-  const int row = b.lo[RA] + sr * kSweepRows - 1 + warp;
-  const int m0 = b.lo[MU] + cm * b.zc, m1 = min(m0 + b.zc, b.hi[MU]);
-  const int s0 = L.s[0], sRA = L.s[RA], sMU = L.s[MU];
-  const int stR = L.st[RA], stM = L.st[MU];
-  const bool pos = (unsigned)x < (unsigned)s0 && (unsigned)row < (unsigned)sRA;
-  const bool owned = warp >= 1 && lane >= HX && lane < HX + OWNX && x < b.hi[0] &&
-                     row < b.hi[RA];
-  const bool xrbox = x >= b.lo[0] && x < b.hi[0] && row >= b.lo[RA] && row < b.hi[RA];
-  const int cxr = x + row * stR;
-  const St<T>* rhoA = (const St<T>*)L.q[F_RHO];
-  const St<T>* eA = (const St<T>*)L.q[F_E];
-  const St<T>* rhoS = kFromB ? (const St<T>*)S.qb[0] : rhoA;
-  const St<T>* eS = kFromB ? (const St<T>*)S.qb[1] : eA;
-  const St<T>* __restrict__ vd = (const St<T>*)L.q[F_VX + d];
-  St<T>* rhoD = kFromB ? (St<T>*)L.q[F_RHO] : (St<T>*)S.qb[0];
-  St<T>* eD = kFromB ? (St<T>*)L.q[F_E] : (St<T>*)S.qb[1];
-  // the momenta are scratch (arithmetic type), rho and e the state type in both copies
-  const C* piA[3] = {(const C*)S.pi[0], (const C*)S.pi[1], (const C*)S.pi[2]};
-  const C* piS[3] = {kFromB ? (const C*)S.qb[2] : piA[0], kFromB ? (const C*)S.qb[3] : piA[1],
-                     kFromB ? (const C*)S.qb[4] : piA[2]};
-  C* piD[3] = {kFromB ? (C*)S.pi[0] : (C*)S.qb[2], kFromB ? (C*)S.pi[1] : (C*)S.qb[3],
-               kFromB ? (C*)S.pi[2] : (C*)S.qb[4]};
-  const C dt = ((const C*)it.dt)[0];
-  const C Adt = it.g.area[d] * dt;
-  const C dtdx = dt * it.g.inv_dx[d];
-  const C F0 = bg.rho0 * bg.V[d] * Adt;
+  const Bg<C> bg = it.bg;
+  const int sM = L.s[d];
+  const unsigned stM = (unsigned)L.st[d] * ES;
+  const unsigned c0 = (unsigned)((EDGE ? min(max(x, 0), L.s[0] - 1) : x) + row * L.st[RA]) * ES;
+  const unsigned cb = EDGE && row < 1 ? c0 : c0 - (unsigned)L.st[RA] * ES;
+  const St<T>* const rhoS = (const St<T>*)(d == 1 ? it.S.F : it.S.P[0]);
+  const St<T>* const eS = (const St<T>*)(d == 1 ? it.S.E : it.S.P[1]);
+  St<T>* const rhoD = (St<T>*)(d == 1 ? it.S.P[0] : L.q[F_RHO]);
+  St<T>* const eD = (St<T>*)(d == 1 ? it.S.P[1] : L.q[F_E]);
+  const St<T>* const vd = (const St<T>*)L.q[F_VX + d];
+  auto piS = [&](int m) { return (const C*)(d == 1 ? it.S.pi[m] : it.S.w[m]); };
+  auto piD = [&](int m) { return (C*)(d == 1 ? it.S.w[m] : it.S.pi[m]); };
+  const C* kc = (const C*)it.kc;
+  const C Adt = kc[K_ADT + d], dtdx = kc[K_DTDX + d];
+  const C F0 = is0(bg.V[d]) ? C(0.f) : kc[K_F0 + d];
   const C iv = it.g.inv_vol;
-  const int sd = L.s[d];
+  const int f0 = L.G, f1 = L.G + L.n[d];
 
-  // state of plane p at this thread's (x, row); zero outside the array
-  auto load = [&](int p, C& r_, C& e_, C& v_, C (&pi_)[3]) {
-    r_ = e_ = v_ = C(0.f);
-    pi_[0] = pi_[1] = pi_[2] = C(0.f);
-    if (pos && (unsigned)p < (unsigned)sMU) {
-      const int c = cxr + p * stM;
-      const bool own = !kFromB || (xrbox && p >= b.lo[MU] && p < b.hi[MU]);
-      r_ = ld(own ? rhoS : rhoA, c);
-      e_ = ld(own ? eS : eA, c);
-      v_ = ld(vd, c);
+  // fetch plane p: this row's values and, of the row below, rho and v_d
+  Ahead<C> ah(buf);
+  const int r_end = m1 + 2;
+  auto fetch = [&](int p) {
+    if (p < r_end && (!EDGE || (unsigned)p < (unsigned)sM)) {
+      const unsigned c = c0 + (unsigned)p * stM, b = cb + (unsigned)p * stM;
+      ah.fetch(0, rhoS, c);
+      ah.fetch(1, eS, c);
+      ah.fetch(2, vd, c);
 #pragma unroll
-      for (int m = 0; m < 3; ++m) pi_[m] = ld(own ? piS[m] : piA[m], c);
+      for (int m = 0; m < 3; ++m) ah.fetch(3 + m, piS(m), c);
+      ah.fetch(6, rhoS, b);
+      ah.fetch(7, vd, b);
     }
+    ah.commit();
   };
-  auto gcoord = [&](int p, int (&g)[3]) {
-    g[0] = x;
-    g[RA] = row;
-    g[MU] = p;
-  };
-  C nr, ne, nv, np[3];
 
-  if constexpr (d != 0) {
-    // ================================================= march along the sweep axis
-    // windows, oldest first, at step r: rho, eps planes r-3..r; e, v_d, Pi planes
-    // r-2..r; w planes r-3..r; F, E faces r-2, r-1; P_d planes r-3, r-2; P_x and
-    // P_row planes r-2, r-1.  The update is of plane r - 2.
-    constexpr int mx = 0, mr = RA;
-    C rw[4] = {}, sw[4] = {}, er[3] = {}, vw[3] = {}, pw[3][3] = {}, ww[3][4] = {};
-    C Fw[2] = {}, Ew[2] = {}, Pd[2] = {}, Pm[2][2] = {};
-    const int nit = m1 - m0 + 5;
-    // Planes far from the array's ends, from the chunk's ends and from a child's
-    // frontier planes pass every test on the plane index; their iterations run a
-    // copy of the body without those tests (FAST), the others the full one.
-    const int r_lo = max(5, m0 + 2), r_hi = min(m1, b.hi[MU] - 2);
-    // state of plane p (inside the box and the array) at this thread's (x, row)
-    auto load_in = [&](int p, C& r_, C& e_, C& v_, C (&pi_)[3]) {
-      r_ = e_ = v_ = C(0.f);
-      pi_[0] = pi_[1] = pi_[2] = C(0.f);
-      if (pos) {
-        const int c = cxr + p * stM;
-        const bool own = !kFromB || xrbox;
-        r_ = ld(own ? rhoS : rhoA, c);
-        e_ = ld(own ? eS : eA, c);
-        v_ = ld(vd, c);
+  // windows at step r (plane r is the newest): x1, x2 the values of planes r-1, r-2, dx0
+  // the difference of planes r and r-1, dx1, dx2 the two before
+  const C z = C(0.f);
+  C r1 = z, r2 = z, dr1 = z, dr2 = z;                       // rho
+  C e1 = z, e2 = z, de1 = z, de2 = z;                       // e/rho
+  C b1 = z, db1 = z, db2 = z, b2 = z;                       // rho, row below
+  C w1[3] = {z, z, z}, w2[3] = {z, z, z};                   // Pi/rho_face - V
+  C dw1[3] = {z, z, z}, dw2[3] = {z, z, z};
+  C en1 = z, en2 = z, v1 = z, v2 = z, vb1 = z;              // e, v_d, v_d of the row below
+  C p1[3] = {z, z, z}, p2[3] = {z, z, z};                   // momenta
+  C F2 = z, E2 = z, Pp[3] = {z, z, z};                      // fluxes of the face before
+  for (int k = 0; k < Ahead<C>::NS - 1; ++k) fetch(m0 - 3 + k);
+#pragma unroll 1
+  for (int r = m0 - 3; r < r_end; ++r) {
+    C q[kSweepArrays];
+    if (sizeof(T) == 8) fetch(r + Ahead<C>::NS - 1);
+    ah.take(q);
+    if (sizeof(T) == 4) fetch(r + 1);
+    C rc = q[0], ec = q[1], vc = q[2], rb = q[6], vb = q[7];
+    C pc[3] = {q[3], q[4], q[5]};
+    if (EDGE && (unsigned)r >= (unsigned)sM)
+      rc = ec = vc = rb = vb = pc[0] = pc[1] = pc[2] = z;
+    // e/rho and Pi/rho_face - V = (dPi - V drf)/(rho0 + drf) of plane r
+    const C ep = eps_dev(ec, rc, bg);
+    const C rx = shfl_up(rc, 1);
+    C w0[3];
 #pragma unroll
-        for (int m = 0; m < 3; ++m) pi_[m] = ld(own ? piS[m] : piA[m], c);
-      }
-    };
-    auto step = [&](int i, auto fast_tag) {
-      constexpr bool FAST = decltype(fast_tag)::value;
-      const int r = m0 - 3 + i;
-      rw[0] = rw[1]; rw[1] = rw[2]; rw[2] = rw[3]; rw[3] = nr;
-      sw[0] = sw[1]; sw[1] = sw[2]; sw[2] = sw[3];
-      sw[3] = eps_dev(ne, nr, bg);
-      er[0] = er[1]; er[1] = er[2]; er[2] = ne;
-      vw[0] = vw[1]; vw[1] = vw[2]; vw[2] = nv;
+    for (int m = 0; m < 3; ++m) {
+      const C drf = halve(add_u(m == 0 ? rx : m == d ? r1 : rb, rc));
+      w0[m] = div_u(sub_ky(pc[m], bg.V[m], drf), add_u(bg.rho0, drf));
+      if (EDGE && !(m == 0 ? x >= 1 : m == d ? r >= 1 && r < sM : row >= 1)) w0[m] = z;
+    }
+    const C dr0 = rc - r1, de0 = ep - e1, db0 = rb - b1;
+    C dw0[3];
 #pragma unroll
-      for (int m = 0; m < 3; ++m) {
-        pw[m][0] = pw[m][1]; pw[m][1] = pw[m][2]; pw[m][2] = np[m];
-      }
-      if (FAST)
-        load_in(r + 1, nr, ne, nv, np);
-      else if (i + 1 < nit)
-        load(r + 1, nr, ne, nv, np);
-      // mass and energy flux of face plane f = r - 1
+    for (int m = 0; m < 3; ++m) dw0[m] = w0[m] - w1[m];
+    C F1 = z, E1 = z;
+    if (r >= m0) {
+      // mass and energy flux of face r - 1, and the mass flux of the row below
       const int f = r - 1;
-      C Fv = C(0.f), Evv = C(0.f);
-      if (pos && (FAST || (f >= 2 && f < sd - 1))) {
-        const C du = vw[1];
-        const C u = bg.V[d] + du;
-        const C cour = u * dtdx;
-        const C drs = upwind_v(rw[0], rw[1], rw[2], rw[3], u, cour);
-        Fv = (bg.rho0 * du + drs * u) * Adt;
-        const C des = upwind_v(sw[0], sw[1], sw[2], sw[3], u, cour);
-        Evv = bg.eps0 * Fv + des * (F0 + Fv);
+      const bool ok = !EDGE || (f >= 2 && f < sM - 1);
+      C Fb = z;
+      if (ok) {
+        const C u = add_k(v1, bg.V[d]), ub = add_k(vb1, bg.V[d]);
+        const C cour = mul_u(u, dtdx);
+        const C drs = upwind_d(r2, r1, dr2, dr1, dr0, u, cour);
+        F1 = mul_u(add_u(mul_u(bg.rho0, v1), mul_u(drs, u)), Adt);  // F - rho0 V_d A dt
+        const C des = upwind_d(e2, e1, de2, de1, de0, u, cour);
+        E1 = add_u(mul_u(bg.eps0, F1), mul_u(des, add_k(F1, F0)));
+        const C drb = upwind_d(b2, b1, db2, db1, db0, ub, mul_u(ub, dtdx));
+        Fb = mul_u(add_u(mul_u(bg.rho0, vb1), mul_u(drb, ub)), Adt);
       }
-      Fw[0] = Fw[1]; Fw[1] = Fv;
-      Ew[0] = Ew[1]; Ew[1] = Evv;
-      if (!FAST && L.is_child && owned && f >= m0 && f < m1 &&
-          (f == L.G || f == L.G + L.n[d])) {
-        // CommFlux record: transverse axes x and the row axis
-        fr_put(L, d, f, x, row, 0, it.sub, as_double(Fv));
-        fr_put(L, d, f, x, row, 1, it.sub, as_double(Evv));
+      if (L.is_child && (f == f0 || f == f1) && own && f >= m0 && (f < m1 || f == it.b.hi[d])) {
+        // CommFlux record (transverse axes x and the row axis): the chunk's own faces
+        // and, above the last chunk, the box's upper face
+        fr_put(L, d, f, x, row, 0, it.sub, as_double(norm(F1)));
+        fr_put(L, d, f, x, row, 1, it.sub, as_double(norm(E1)));
       }
-      // rho_r, v_{r-1}, F_{r-1} of the row below (shared) and of x - 1 (shuffle)
-      C* xb = xch + (i & 1) * 3 * NT;
-      xb[tid] = rw[3];
-      xb[NT + tid] = vw[1];
-      xb[2 * NT + tid] = Fv;
-      __syncthreads();
-      if (warp == 0) return;  // the halo row only supplies rho, v_d and F
-      const C r_rb = xb[tid - 32], v_rb = xb[NT + tid - 32], F_rb = xb[2 * NT + tid - 32];
-      const C r_xb = shfl_up(rw[3], 1), v_xb = shfl_up(vw[1], 1), F_xb = shfl_up(Fv, 1);
-      // w = (dPi - V drf) / (rho0 + drf) of plane r
-      const bool pok = pos && (FAST || (unsigned)r < (unsigned)sMU);
-#pragma unroll
-      for (int m = 0; m < 3; ++m) {
-        const C rn = m == mx ? r_xb : (m == mr ? r_rb : rw[2]);
-        const bool g1 = m == mx ? x >= 1 : (m == mr ? row >= 1 : (FAST || r >= 1));
-        C wv = C(0.f);
-        if (pok && g1) {
-          const C drf = halve(rn + rw[3]);
-          wv = hdiv(pw[m][2] - bg.V[m] * drf, bg.rho0 + drf);
+      const C Fx = shfl_up(F1, 1), vx = shfl_up(v1, 1);
+      C P[3] = {z, z, z};
+      if (r >= m0 + 1) {
+        // momentum fluxes: on the x and row edges of plane r - 1, along d at cell r - 2
+        if (!EDGE || (ok && x >= 1)) {
+          const C ue = add_k(halve(vx + v1), bg.V[d]);
+          const C Fe = halve(add_u(Fx, F1));
+          const C ws = upwind_d(w2[0], w1[0], dw2[0], dw1[0], dw0[0], ue, mul_u(ue, dtdx));
+          P[0] = ky_add(bg.V[0], Fe, mul_u(ws, add_k(Fe, F0)));
         }
-        ww[m][0] = ww[m][1]; ww[m][1] = ww[m][2]; ww[m][2] = ww[m][3]; ww[m][3] = wv;
-      }
-      // P_x, P_row of plane q = r - 1 (d-m edges)
-      const int q = r - 1;
-#pragma unroll
-      for (int j = 0; j < 2; ++j) {
-        const int m = j == 0 ? mx : mr;
-        C P = C(0.f);
-        if (pos && (FAST || (q >= 2 && q < sd - 1)) && (j == 0 ? x >= 1 : row >= 1)) {
-          const C ue = bg.V[d] + halve((j == 0 ? v_xb : v_rb) + vw[1]);
-          const C Fe = halve((j == 0 ? F_xb : F_rb) + Fv);
-          const C wsv = upwind_v(ww[m][0], ww[m][1], ww[m][2], ww[m][3], ue, ue * dtdx);
-          P = bg.V[m] * Fe + wsv * (F0 + Fe);
+        if (!EDGE || (ok && row >= 1)) {
+          const C ue = add_k(halve(vb1 + v1), bg.V[d]);
+          const C Fe = halve(add_u(Fb, F1));
+          const C ws = upwind_d(w2[RA], w1[RA], dw2[RA], dw1[RA], dw0[RA], ue, mul_u(ue, dtdx));
+          P[RA] = ky_add(bg.V[RA], Fe, mul_u(ws, add_k(Fe, F0)));
         }
-        Pm[j][0] = Pm[j][1];
-        Pm[j][1] = P;
-      }
-      // P_d of plane p = r - 2 (cell-centred)
-      {
-        const int p = r - 2;
-        C P = C(0.f);
-        if (pos && (FAST || (p >= 2 && p < sd - 2))) {
-          const C uc = bg.V[d] + halve(vw[0] + vw[1]);
-          const C Fc = halve(Fw[0] + Fw[1]);
-          const C wsv = upwind_v(ww[d][0], ww[d][1], ww[d][2], ww[d][3], uc, uc * dtdx);
-          P = bg.V[d] * Fc + wsv * (F0 + Fc);
+        if (!EDGE || (r - 2 >= 2 && r - 2 < sM - 2)) {
+          const C uc = add_k(halve(v2 + v1), bg.V[d]);
+          const C Fc = halve(add_u(F2, F1));
+          const C ws = upwind_d(w2[d], w1[d], dw2[d], dw1[d], dw0[d], uc, mul_u(uc, dtdx));
+          P[d] = ky_add(bg.V[d], Fc, mul_u(ws, add_k(Fc, F0)));
         }
-        Pd[0] = Pd[1];
-        Pd[1] = P;
       }
-      // conservative update of plane u = r - 2
-      const int u = r - 2;
-      if (owned && (FAST || (u >= m0 && u < m1))) {
-        const int c = cxr + u * stM;
-        C rv = rw[1], evv = er[0];
-        if (FAST || (u >= 2 && u < sd - 2)) {
-          C Flo = Fw[0], Fhi = Fw[1], Elo = Ew[0], Ehi = Ew[1];
-          if (!FAST && L.has_child) {
+      // conservative update of plane r - 2
+      const int u2 = r - 2;
+      if (u2 >= m0 && own) {
+        const unsigned c = c0 + (unsigned)u2 * stM;
+        const bool upd = !EDGE || (u2 >= 2 && u2 < sM - 2);
+        C rv = r2, ev = en2;
+        if (upd) {
+          C Flo = F2, Fhi = F1, Elo = E2, Ehi = E1;
+          if (L.has_child && near_frontier(L, d, u2)) {
             int g[3];
-            gcoord(u, g);
+            g[0] = x;
+            g[RA] = row;
+            g[d] = u2;
             frontier_fluxes(L, d, g, Flo, Fhi, Elo, Ehi);
           }
-          rv = rv - (Fhi - Flo) * iv;
-          evv = evv - (Ehi - Elo) * iv;
+          rv = rv - mul_u(sub_u(Fhi, Flo), iv);
+          ev = ev - mul_u(sub_u(Ehi, Elo), iv);
         }
-        st(rhoD, c, rv);
-        st(eD, c, evv);
+        stb(rhoD, c, rv);
+        stb(eD, c, ev);
 #pragma unroll
         for (int m = 0; m < 3; ++m) {
-          C pv = pw[m][0];
-          if (m == d) {
-            if (FAST || (u >= 3 && u < sd - 2)) pv = pv - (Pd[1] - Pd[0]) * iv;
-          } else {
-            const int j = m == mx ? 0 : 1;
-            if ((FAST || (u >= 2 && u < sd - 2)) && (j == 0 ? x >= 1 : row >= 1))
-              pv = pv - (Pm[j][1] - Pm[j][0]) * iv;
-          }
-          st(piD[m], c, pv);
+          C pv = p2[m];
+          // P_d of cells r-3, r-2; the others' of planes r-2, r-1
+          if (!EDGE || (upd && (m == d ? u2 >= 3 : m == 0 ? x >= 1 : row >= 1)))
+            pv = sub_u(pv, mul_u(sub_u(P[m], Pp[m]), iv));
+          stb(piD(m), c, pv);
         }
       }
-    };
-    load(m0 - 3, nr, ne, nv, np);
-    for (int i = 0; i < nit; ++i) {
-      const int r = m0 - 3 + i;
-      const bool fast = r >= r_lo && r <= r_hi &&
-                        !(L.is_child && (r - 1 == L.G || r - 1 == L.G + L.n[d])) &&
-                        !(L.has_child && near_frontier(L, d, r - 2));
-      if (fast)
-        step(i, std::true_type{});
-      else
-        step(i, std::false_type{});
+#pragma unroll
+      for (int m = 0; m < 3; ++m) Pp[m] = P[m];
     }
-  } else {
-    // ======================================================== x sweep, march in z
-    C pr_r = C(0.f), pr_v = C(0.f), pr_F = C(0.f);  // plane r - 1 at (x, row)
-    const int nit = m1 - m0 + 1;
-    load(m0 - 1, nr, ne, nv, np);
-    for (int i = 0; i < nit; ++i) {
-      const int r = m0 - 1 + i;
-      const C rc = nr, ec = ne, vc = nv, pi0 = np[0], pi1 = np[1], pi2 = np[2];
-      if (i + 1 < nit) load(r + 1, nr, ne, nv, np);
+    F2 = F1; E2 = E1;
+    r2 = r1; r1 = rc; dr2 = dr1; dr1 = dr0;
+    e2 = e1; e1 = ep; de2 = de1; de1 = de0;
+    b2 = b1; b1 = rb; db2 = db1; db1 = db0;
+    en2 = en1; en1 = ec; v2 = v1; v1 = vc; vb1 = vb;
+#pragma unroll
+    for (int m = 0; m < 3; ++m) {
+      w2[m] = w1[m]; w1[m] = w0[m]; dw2[m] = dw1[m]; dw1[m] = dw0[m];
+      p2[m] = p1[m]; p1[m] = pc[m];
+    }
+  }
+}
+
+// the x sweep
+template <class T, bool EDGE>
+__device__ __forceinline__ void sweep_x(const Item<T>& it, int x, int row, bool mine, int m0,
+                                        int m1, Arith<T>* __restrict__ buf) {
+  using C = Arith<T>;
+  constexpr unsigned ES = sizeof(C);
+  const LevelView& L = it.L;
+  const Bg<C> bg = it.bg;
+  const bool own = mine && x >= it.b.lo[0] && x < it.b.hi[0];
+  const int sx = L.s[0];
+  const unsigned stM = (unsigned)L.st[2] * ES;
+  const unsigned c0 = (unsigned)((EDGE ? min(max(x, 0), sx - 1) : x) + row * L.st[1]) * ES;
+  const unsigned cb = EDGE && row < 1 ? c0 : c0 - (unsigned)L.st[1] * ES;
+  const St<T>* const rhoS = (const St<T>*)L.q[F_RHO];
+  const St<T>* const eS = (const St<T>*)L.q[F_E];
+  const C* kc = (const C*)it.kc;
+  const C Adt = kc[K_ADT], dtdx = kc[K_DTDX];
+  const C F0 = is0(bg.V[0]) ? C(0.f) : kc[K_F0];
+  const C iv = it.g.inv_vol;
+  // CommFlux record: the box's own faces and its upper one
+  const bool rec = L.is_child && mine && (x == L.G || x == L.G + L.n[0]) &&
+                   x >= it.b.lo[0] && x <= it.b.hi[0];
+  const bool near = L.has_child && near_frontier(L, 0, x);
+  const bool okF = !EDGE || (x >= 2 && x < sx - 1);
+  const C z = C(0.f);
+
+  Ahead<C> ah(buf);
+  auto fetch = [&](int p) {
+    if (p < m1 && (!EDGE || p >= 0)) {
+      const unsigned c = c0 + (unsigned)p * stM, b = cb + (unsigned)p * stM;
+      ah.fetch(0, rhoS, c);
+      ah.fetch(1, eS, c);
+#pragma unroll
+      for (int m = 0; m < 3; ++m) ah.fetch(2 + m, (const St<T>*)L.q[F_VX + m], c);
+      ah.fetch(5, rhoS, b);
+      ah.fetch(6, (const St<T>*)L.q[F_VX], b);
+    }
+    ah.commit();
+  };
+  for (int k = 0; k < Ahead<C>::NS - 1; ++k) fetch(m0 - 1 + k);
+  C rp = z, vp = z, Fp = z;  // rho, v_x, F of the plane before
+#pragma unroll 1
+  for (int p = m0 - 1; p < m1; ++p) {
+    C q[kSweepArrays];
+    if (sizeof(T) == 8) fetch(p + Ahead<C>::NS - 1);
+    ah.take(q);
+    if (sizeof(T) == 4) fetch(p + 1);
+    C rc = q[0], ec = q[1], rb = q[5], vb = q[6];
+    C w[3] = {q[2], q[3], q[4]};
+    if (EDGE && p < 0) rc = ec = rb = vb = w[0] = w[1] = w[2] = z;
+    const C vc = w[0];
+    const C r_m1 = shfl_up(rc, 1);
+    C Fv = z, Ev = z, Fb = z;
+    {
+      // each lane forms its difference to the lane below, the neighbours read it
       const C ep = eps_dev(ec, rc, bg);
-      const C r_m2 = shfl_up(rc, 2), r_m1 = shfl_up(rc, 1), r_p1 = shfl_dn(rc, 1);
-      const C e_m2 = shfl_up(ep, 2), e_m1 = shfl_up(ep, 1), e_p1 = shfl_dn(ep, 1);
-      const bool pok = pos && (unsigned)r < (unsigned)sMU;
-      // mass and energy flux at the x-face of this cell
-      C Fv = C(0.f), Evv = C(0.f);
-      if (pok && x >= 2 && x < sd - 1) {
-        const C u = bg.V[0] + vc;
-        const C cour = u * dtdx;
-        const C drs = upwind_v(r_m2, r_m1, rc, r_p1, u, cour);
-        Fv = (bg.rho0 * vc + drs * u) * Adt;
-        const C des = upwind_v(e_m2, e_m1, ep, e_p1, u, cour);
-        Evv = bg.eps0 * Fv + des * (F0 + Fv);
+      const C e_m1 = shfl_up(ep, 1), b_m1 = shfl_up(rb, 1);
+      const C dr = rc - r_m1, de = ep - e_m1, db = rb - b_m1;
+      const C dr_m = shfl_up(dr, 1), dr_p = shfl_dn(dr, 1);
+      const C de_m = shfl_up(de, 1), de_p = shfl_dn(de, 1);
+      const C db_m = shfl_up(db, 1), db_p = shfl_dn(db, 1);
+      if (!EDGE || (okF && p >= 0)) {
+        const C u = add_k(vc, bg.V[0]), ub = add_k(vb, bg.V[0]);
+        const C cour = mul_u(u, dtdx);
+        const C drs = upwind_d(r_m1, rc, dr_m, dr, dr_p, u, cour);
+        Fv = mul_u(add_u(mul_u(bg.rho0, vc), mul_u(drs, u)), Adt);  // F - rho0 V_x A dt
+        const C des = upwind_d(e_m1, ep, de_m, de, de_p, u, cour);
+        Ev = add_u(mul_u(bg.eps0, Fv), mul_u(des, add_k(Fv, F0)));
+        const C drb = upwind_d(b_m1, rb, db_m, db, db_p, ub, mul_u(ub, dtdx));
+        Fb = mul_u(add_u(mul_u(bg.rho0, vb), mul_u(drb, ub)), Adt);
       }
-      if (L.is_child && owned && r >= m0 && r < m1 && (x == L.G || x == L.G + L.n[0])) {
-        // CommFlux record: transverse axes y (the row) and z (the march)
-        fr_put(L, 0, x, row, r, 0, it.sub, as_double(Fv));
-        fr_put(L, 0, x, row, r, 1, it.sub, as_double(Evv));
-      }
-      // rho, v_x, F of the row below
-      C* xb = xch + (i & 1) * 3 * NT;
-      xb[tid] = rc;
-      xb[NT + tid] = vc;
-      xb[2 * NT + tid] = Fv;
-      __syncthreads();
-      // plane m0 - 1 only feeds the z-fluxes of plane m0; the halo row only supplies
-      // rho, v_x and F
-      if (i > 0 && warp > 0) {
-        const C r_rb = xb[tid - 32], v_rb = xb[NT + tid - 32], F_rb = xb[2 * NT + tid - 32];
-        // w of this plane: along x (lane below), y (row below), z (previous plane)
-        C wx = C(0.f), wy = C(0.f), wz = C(0.f);
-        if (pok && x >= 1) {
-          const C drf = halve(r_m1 + rc);
-          wx = hdiv(pi0 - bg.V[0] * drf, bg.rho0 + drf);
-        }
-        if (pok && row >= 1) {
-          const C drf = halve(r_rb + rc);
-          wy = hdiv(pi1 - bg.V[1] * drf, bg.rho0 + drf);
-        }
-        if (pok && r >= 1) {
-          const C drf = halve(pr_r + rc);
-          wz = hdiv(pi2 - bg.V[2] * drf, bg.rho0 + drf);
-        }
-        const C wx_m1 = shfl_up(wx, 1), wx_p1 = shfl_dn(wx, 1), wx_p2 = shfl_dn(wx, 2);
-        const C wy_m2 = shfl_up(wy, 2), wy_m1 = shfl_up(wy, 1), wy_p1 = shfl_dn(wy, 1);
-        const C wz_m2 = shfl_up(wz, 2), wz_m1 = shfl_up(wz, 1), wz_p1 = shfl_dn(wz, 1);
-        const C v_p1 = shfl_dn(vc, 1), F_p1 = shfl_dn(Fv, 1), E_p1 = shfl_dn(Evv, 1);
-        // momentum fluxes: P_x cell-centred, P_y and P_z on the x-y and x-z edges
-        C Px = C(0.f), Py = C(0.f), Pz = C(0.f);
-        if (pok && x >= 2 && x < sd - 2) {
-          const C uc = bg.V[0] + halve(vc + v_p1);
-          const C Fc = halve(Fv + F_p1);
-          const C wsv = upwind_v(wx_m1, wx, wx_p1, wx_p2, uc, uc * dtdx);
-          Px = bg.V[0] * Fc + wsv * (F0 + Fc);
-        }
-        if (pok && x >= 2 && x < sd - 1 && row >= 1) {
-          const C ue = bg.V[0] + halve(v_rb + vc);
-          const C Fe = halve(F_rb + Fv);
-          const C wsv = upwind_v(wy_m2, wy_m1, wy, wy_p1, ue, ue * dtdx);
-          Py = bg.V[1] * Fe + wsv * (F0 + Fe);
-        }
-        if (pok && x >= 2 && x < sd - 1 && r >= 1) {
-          const C ue = bg.V[0] + halve(pr_v + vc);
-          const C Fe = halve(pr_F + Fv);
-          const C wsv = upwind_v(wz_m2, wz_m1, wz, wz_p1, ue, ue * dtdx);
-          Pz = bg.V[2] * Fe + wsv * (F0 + Fe);
-        }
-        const C Px_m1 = shfl_up(Px, 1), Py_p1 = shfl_dn(Py, 1), Pz_p1 = shfl_dn(Pz, 1);
-        // conservative update of this cell
-        if (owned && r >= m0 && r < m1) {
-          const int c = cxr + r * stM;
-          C rv = rc, evv = ec;
-          if (x >= 2 && x < sd - 2) {
-            C Flo = Fv, Fhi = F_p1, Elo = Evv, Ehi = E_p1;
-            if (L.has_child) {
-              int g[3];
-              gcoord(r, g);
-              frontier_fluxes(L, 0, g, Flo, Fhi, Elo, Ehi);
-            }
-            rv = rv - (Fhi - Flo) * iv;
-            evv = evv - (Ehi - Elo) * iv;
-          }
-          st(rhoD, c, rv);
-          st(eD, c, evv);
-          C p0 = pi0, p1 = pi1, p2 = pi2;
-          if (x >= 3 && x < sd - 2) p0 = p0 - (Px - Px_m1) * iv;
-          if (x >= 2 && x < sd - 2 && row >= 1) p1 = p1 - (Py_p1 - Py) * iv;
-          if (x >= 2 && x < sd - 2 && r >= 1) p2 = p2 - (Pz_p1 - Pz) * iv;
-          st(piD[0], c, p0);
-          st(piD[1], c, p1);
-          st(piD[2], c, p2);
-        }
-      }
-      pr_r = rc;
-      pr_v = vc;
-      pr_F = Fv;
     }
+    if (p >= m0) {
+      if (rec) {  // transverse axes y and z
+        fr_put(L, 0, x, row, p, 0, it.sub, as_double(norm(Fv)));
+        fr_put(L, 0, x, row, p, 1, it.sub, as_double(norm(Ev)));
+      }
+      const C F_p1 = shfl_dn(Fv, 1), E_p1 = shfl_dn(Ev, 1), v_p1 = shfl_dn(vc, 1);
+      // momentum fluxes: P_x cell-centred, P_y and P_z on the x-y and x-z edges
+      C P[3] = {z, z, z};
+      {
+        const C dw = w[0] - shfl_up(w[0], 1);
+        const C dw_p = shfl_dn(dw, 1), dw_p2 = shfl_dn(dw, 2);
+        if (!EDGE || (x >= 2 && x < sx - 2)) {
+          const C uc = add_k(halve(vc + v_p1), bg.V[0]);
+          const C Fc = halve(add_u(Fv, F_p1));
+          const C ws = upwind_d(w[0], v_p1, dw, dw_p, dw_p2, uc, mul_u(uc, dtdx));
+          P[0] = ky_add(bg.V[0], Fc, mul_u(ws, add_k(Fc, F0)));
+        }
+      }
+#pragma unroll
+      for (int m = 1; m < 3; ++m) {
+        const C w_m1 = shfl_up(w[m], 1), dw = w[m] - w_m1;
+        const C dw_m = shfl_up(dw, 1), dw_p = shfl_dn(dw, 1);
+        if (!EDGE || (okF && (m == 1 ? row >= 1 : p >= 1))) {
+          const C ue = add_k(halve((m == 1 ? vb : vp) + vc), bg.V[0]);
+          const C Fe = halve(add_u(m == 1 ? Fb : Fp, Fv));
+          const C ws = upwind_d(w_m1, w[m], dw_m, dw, dw_p, ue, mul_u(ue, dtdx));
+          P[m] = ky_add(bg.V[m], Fe, mul_u(ws, add_k(Fe, F0)));
+        }
+      }
+      const C Px_m1 = shfl_up(P[0], 1), Py_p1 = shfl_dn(P[1], 1), Pz_p1 = shfl_dn(P[2], 1);
+      // conservative update of this cell
+      if (own) {
+        const unsigned c = c0 + (unsigned)p * stM;
+        const bool upd = !EDGE || (x >= 2 && x < sx - 2);
+        C rv = rc, ev = ec;
+        if (upd) {
+          C Flo = Fv, Fhi = F_p1, Elo = Ev, Ehi = E_p1;
+          if (near) {
+            const int g[3] = {x, row, p};
+            frontier_fluxes(L, 0, g, Flo, Fhi, Elo, Ehi);
+          }
+          rv = rv - mul_u(sub_u(Fhi, Flo), iv);
+          ev = ev - mul_u(sub_u(Ehi, Elo), iv);
+        }
+        stb((St<T>*)it.S.F, c, rv);
+        stb((St<T>*)it.S.E, c, ev);
+#pragma unroll
+        for (int m = 0; m < 3; ++m) {
+          C pv = z;  // the momentum Pi - rho0 V of v
+          const bool in = !EDGE || (m == 0 ? x >= 1 : m == 1 ? row >= 1 : p >= 1);
+          if (in) {
+            const C drf = halve(add_u(m == 0 ? r_m1 : m == 1 ? rb : rp, rc));
+            pv = add_u(mul_u(bg.rho0, w[m]), mul_u(drf, add_k(w[m], bg.V[m])));
+          }
+          if (!EDGE || (upd && in && (m != 0 || x >= 3)))
+            pv = sub_u(pv, mul_u(m == 0 ? sub_u(P[0], Px_m1) : sub_u(m == 1 ? Py_p1 : Pz_p1, P[m]), iv));
+          stb((C*)it.S.pi[m], c, pv);
+        }
+      }
+    }
+    rp = rc;
+    vp = vc;
+    Fp = Fv;
+  }
+}
+
+template <class T, int d>
+__device__ __forceinline__ void el_sweep(const Item<T>& it, unsigned unit,
+                                         Arith<T>* __restrict__ buf) {
+  constexpr int RA = d == 1 ? 2 : 1, MU = d == 0 ? 2 : d;
+  const Box& b = it.b;
+  const int ncol = sweep_columns(b, d);
+  const int chunk = (int)unit / ncol, col = (int)unit - chunk * ncol;
+  SweepLane p;
+  if (!sweep_lane(b, d, col * (kSweepThreads / 32) + (int)(threadIdx.x >> 5),
+                  (int)(threadIdx.x & 31), p))
+    return;
+  const int m0 = b.lo[MU] + chunk * b.zc, m1 = min(m0 + b.zc, b.hi[MU]);
+  if (d == 0) {
+    if (b.lo[0] >= 3 && b.hi[0] <= it.L.s[0] - 2 && b.lo[1] >= 1 && m0 >= 1)
+      sweep_x<T, false>(it, p.x, p.row, p.mine, m0, m1, buf);
+    else
+      sweep_x<T, true>(it, p.x, p.row, p.mine, m0, m1, buf);
+  } else {
+    if (b.lo[0] >= 1 && b.lo[RA] >= 1 && m0 >= 3 && m1 <= it.L.s[d] - 2)
+      sweep_march<T, d == 0 ? 1 : d, false>(it, p.x, p.row, p.mine && p.x >= b.lo[0], m0, m1, buf);
+    else
+      sweep_march<T, d == 0 ? 1 : d, true>(it, p.x, p.row, p.mine && p.x >= b.lo[0], m0, m1, buf);
   }
 }
 
@@ -1181,7 +1261,7 @@ template <class T, int NC, int KICK2>
 __device__ __forceinline__ void el_vrec_source(const LevelView& L, const Box& b, const Scratch& S,
                                                const Arith<T>* __restrict__ dtp, Arith<T> gm1,
                                                const Bg<Arith<T>>& bg, const Geo<Arith<T>>& g,
-                                               int fused, int write_pi, const unsigned* el) {
+                                               int write_pi, const unsigned* el) {
   using C = Arith<T>;
   int c[NC], c3[NC][3];
   bool ok[NC];
@@ -1196,20 +1276,13 @@ __device__ __forceinline__ void el_vrec_source(const LevelView& L, const Box& b,
     c3[n][1] = j;
     c3[n][2] = k;
   }
-  St<T>* rhoA = (St<T>*)L.q[F_RHO];
-  St<T>* eA = (St<T>*)L.q[F_E];
-  // after fused sweeps the box's state is in Scratch::qb; outside the box it is in
-  // the level's arrays, which this op then updates for the box
-  const St<T>* rho = fused ? (const St<T>*)S.qb[0] : rhoA;
-  const St<T>* e = fused ? (const St<T>*)S.qb[1] : eA;
+  const St<T>* __restrict__ rho = (const St<T>*)L.q[F_RHO];
+  const St<T>* __restrict__ e = (const St<T>*)L.q[F_E];
   const Arith<T>* __restrict__ phi = (const Arith<T>*)L.phi;
   const C h = halve(dtp[0]);
-  St<T> rc_s[NC], ec_s[NC];
   C rc[NC], ec[NC], fc[NC], rm[NC][3], em[NC][3], fm[NC][3], pv[NC][3];
 #pragma unroll
   for (int n = 0; n < NC; ++n) {
-    rc_s[n] = rho[c[n]];
-    ec_s[n] = e[c[n]];
     rc[n] = ld(rho, c[n]);
     ec[n] = ld(e, c[n]);
     fc[n] = ld(phi, c[n]);
@@ -1217,11 +1290,10 @@ __device__ __forceinline__ void el_vrec_source(const LevelView& L, const Box& b,
     for (int d = 0; d < 3; ++d)
       if (c3[n][d] >= 1) {
         const int m = c[n] - L.st[d];
-        const bool own = !fused || c3[n][d] - 1 >= b.lo[d];
-        rm[n][d] = ld(own ? rho : (const St<T>*)rhoA, m);
-        em[n][d] = ld(own ? e : (const St<T>*)eA, m);
+        rm[n][d] = ld(rho, m);
+        em[n][d] = ld(e, m);
         fm[n][d] = ld(phi, m);
-        pv[n][d] = ld((const C*)(fused ? S.qb[2 + d] : S.pi[d]), c[n]);
+        pv[n][d] = ld((const C*)S.pi[d], c[n]);
       }
   }
 #pragma unroll
@@ -1248,10 +1320,6 @@ __device__ __forceinline__ void el_vrec_source(const LevelView& L, const Box& b,
           st((Arith<T>*)S.pi[d], c[n], mul_u(bg.rho0, vn) + mul_u(drf, add_k(vn, bg.V[d])));
       }
       st((St<T>*)L.q[F_VX + d], c[n], vn);
-    }
-    if (fused) {
-      rhoA[c[n]] = rc_s[n];
-      eA[c[n]] = ec_s[n];
     }
   }
 }
@@ -2169,7 +2237,7 @@ __device__ __forceinline__ void run_op(const Item<T>& it, unsigned tid) {
     el_visc_v<T>(it.L, it.b, it.S, (const Arith<T>*)it.dt, it.flags & FL_WRITE_PI, it.bg, it.g, tid);
   else if (OP == OP_VREC)  // D = 1: with the next sub-cycle's first kick
     el_vrec_source<T, NC, D>(it.L, it.b, it.S, (const Arith<T>*)it.dt, it.gm1, it.bg, it.g,
-                             it.flags & FL_FUSED, it.flags & FL_WRITE_PI, el);
+                             it.flags & FL_WRITE_PI, el);
   else if (OP == OP_BC)
     el_bc_axis<T>(it.L, D, it.bc_lo, it.bc_hi, (T)it.V[0], (T)it.V[1], (T)it.V[2], tid);
   else if (OP == OP_COMMUP)
@@ -2247,22 +2315,23 @@ __global__ void __launch_bounds__(kBlock) k_single(const Item<T> it) {
   pdl_exit();
 }
 
-// Fused sweep: one block per (column, chunk) unit; the work-list form stages the
-// item as k_batch does.
+// Fused sweep: one block per (column, chunk) unit; the work-list form stages the item as
+// k_batch does.
 template <class T, int D>
-__global__ void __launch_bounds__(kSweepThreads) k_sweep_single(const Item<T> it) {
-  __shared__ __align__(16) Arith<T> s_x[2 * 3 * kSweepThreads];
+__global__ void __launch_bounds__(kSweepThreads, sweep_blocks((int)sizeof(T), D))
+    k_sweep_single(const Item<T> it) {
+  __shared__ Arith<T> s_ahead[sweep_ahead((int)sizeof(T))];
   pdl_enter();
   if (skipped(it)) return;
-  el_sweep<T, D>(it, blockIdx.x, s_x);
+  el_sweep<T, D>(it, blockIdx.x, s_ahead + threadIdx.x);
   pdl_exit();
 }
 
 template <class T, int D>
-__global__ void __launch_bounds__(kSweepThreads, sizeof(T) == 4 ? 2 : 1) k_sweep_batch(const Item<T>* __restrict__ items,
-                                                              const unsigned* __restrict__ starts,
-                                                              int nitems, unsigned nchunks) {
-  __shared__ __align__(16) Arith<T> s_x[2 * 3 * kSweepThreads];
+__global__ void __launch_bounds__(kSweepThreads, sweep_blocks((int)sizeof(T), D))
+    k_sweep_batch(const Item<T>* __restrict__ items, const unsigned* __restrict__ starts,
+                  int nitems, unsigned nchunks) {
+  __shared__ Arith<T> s_ahead[sweep_ahead((int)sizeof(T))];
   __shared__ __align__(16) unsigned char s_raw[sizeof(Item<T>)];
   const Item<T>& it = *reinterpret_cast<const Item<T>*>(s_raw);
   pdl_enter();
@@ -2287,7 +2356,7 @@ __global__ void __launch_bounds__(kSweepThreads, sizeof(T) == 4 ? 2 : 1) k_sweep
       __syncthreads();
       cur = lo;
     }
-    if (!skipped(it)) el_sweep<T, D>(it, ch - starts[cur], s_x);
+    if (!skipped(it)) el_sweep<T, D>(it, ch - starts[cur], s_ahead + threadIdx.x);
     __syncthreads();
   }
   pdl_exit();
@@ -2296,8 +2365,8 @@ __global__ void __launch_bounds__(kSweepThreads, sizeof(T) == 4 ? 2 : 1) k_sweep
 // launch with the programmatic-stream-serialisation attribute (see pdl_enter); an
 // error is left in the runtime's last-error state like that of a <<<>>> launch
 template <class... P, class... A>
-static void launch_pdl(void (*kernel)(P...), unsigned grid, unsigned block, cudaStream_t st,
-                       A&&... args) {
+static void launch_pdl(void (*kernel)(P...), unsigned grid, unsigned block,
+                       cudaStream_t st, A&&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);
   cfg.blockDim = dim3(block);
@@ -2382,34 +2451,6 @@ int launch_batch(int op, int d, const Item<T>* items, const unsigned* starts, in
 #undef DFN_OP
 #undef DFN_OPD
   return 1;
-}
-
-// blocks of a context's sweep kernel to aim for: those resident on the whole device
-// at once (SMs x the blocks one SM holds), per state size and direction; looked up
-// once
-int sweep_slots(int esz, int d) {
-  static int cache[2][3] = {};
-  const int t = esz == 8 ? 1 : 0;
-  if (cache[t][d] == 0) {
-    int dev = 0, sms = 0, per = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const void* k = nullptr;
-    if (esz == 8)
-      k = d == 0 ? (const void*)k_sweep_single<double, 0>
-                 : d == 1 ? (const void*)k_sweep_single<double, 1>
-                          : (const void*)k_sweep_single<double, 2>;
-    else
-      k = d == 0 ? (const void*)k_sweep_single<float, 0>
-                 : d == 1 ? (const void*)k_sweep_single<float, 1>
-                          : (const void*)k_sweep_single<float, 2>;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, kSweepThreads, 0) != cudaSuccess)
-      per = 1;
-    // with a single resident block per SM, several waves hide latency better than
-    // long chunks (measured on the FP64 state's sweeps): keep about 600 blocks
-    cache[t][d] = per >= 2 ? sms * per : 600;
-  }
-  return cache[t][d];
 }
 
 // elements per chunk of each op (one chunk = one block pass)
