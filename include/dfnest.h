@@ -232,8 +232,7 @@ int df_set_tile_shapes(df_ctx* ctx, const int* shapes);
  * memory traffic.  The two give the same arithmetic on every active cell up to rounding
  * (the compiler's contraction of multiply-adds; at the x sweep the fused form forms the
  * momenta from v and rho; in double-float it leaves more intermediate sums
- * unnormalised).  DF_TRANSPORT_AUTO (default): separate for DF_FP64, fused for
- * DF_FP32_STATE. */
+ * unnormalised).  DF_TRANSPORT_AUTO (default): fused. */
 #define DF_TRANSPORT_AUTO 0
 #define DF_TRANSPORT_SEPARATE 1
 #define DF_TRANSPORT_FUSED 2

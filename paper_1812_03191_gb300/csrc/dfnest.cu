@@ -555,13 +555,87 @@ struct TileTable {
   }
 };
 
-// Transport of one level step: DF_TRANSPORT_FUSED or DF_TRANSPORT_SEPARATE as set;
-// DF_TRANSPORT_AUTO takes the fused sweeps for the FP32 state (against the separate
-// kernels, per coarse step: 3 x 64^3 0.47 to 0.59 ms, nine quadrant levels of 32x32x64
-// 27.8 to 32.1) and the separate kernels for FP64 (nine quadrant levels 41.4 to 44.4).
-bool sweeps_fused(int mode, int prec) {
-  if (mode != DF_TRANSPORT_AUTO) return mode == DF_TRANSPORT_FUSED;
-  return prec == DF_FP32_STATE;
+// Element range per axis, [lo, hi), of a padded array.
+struct Range {
+  int lo[3], hi[3];
+  // with `below` more elements under it and `above` over it along axis d
+  Range grown(int d, int below, int above) const {
+    Range r = *this;
+    r.lo[d] -= below;
+    r.hi[d] += above;
+    return r;
+  }
+  void cover(const Range& o) {
+    for (int d = 0; d < 3; ++d) {
+      lo[d] = std::min(lo[d], o.lo[d]);
+      hi[d] = std::max(hi[d], o.hi[d]);
+    }
+  }
+};
+
+// Elements that have to be right at some point of a level step: rho and e, and each
+// velocity component.
+struct Need {
+  Range re, v[3];
+};
+
+// The box of every op of one level step (fused sweeps), and what it needs of the state
+// before it.
+struct StepBoxes {
+  Range source, compress, diffuse, sweep[3], vrec;
+  Need before;
+};
+
+// The boxes that give `after` at the end of a level step, from the stencils, last op
+// first.  Sweeping the active cells +- 8 and +- 4 with every op instead did 1.14 times
+// (128^3) to 1.5 times (32^3) the work.
+//   velocity recovery and kick: v_d of c from rho, e of c-1, c along d and Pi_d of c;
+//   sweep along d: rho, e of c from rho, e of c-2..c+2 and v_d of c, c+1; Pi_d of c from
+// Pi_d of c-2..c+2, rho, e of c-3..c+2 and v_d of c-1..c+1; Pi_m of c from Pi_m of
+// c-2..c+2 along d, and from rho, e of the same and v_d of c, c+1, there and one below
+// along m; the x sweep reads velocities in place of momenta;
+//   diffusion: e of c from rho, e/rho of c-1..c+1 along each axis; compression: e of c
+// from v_d of c, c+1 along d; first kick: v_d of c from rho, e of c-1, c along d.
+StepBoxes step_boxes(const Need& after, bool hydro, bool diffusion) {
+  StepBoxes b;
+  Range re = after.re, pi[3], v[3];
+  if (hydro) {
+    b.vrec = after.v[0];
+    for (int d = 0; d < 3; ++d) {
+      b.vrec.cover(after.v[d]);
+      pi[d] = after.v[d];
+      re.cover(after.v[d].grown(d, 1, 0));
+    }
+    for (int d = 2; d >= 0; --d) {
+      Range out = re, in = re.grown(d, 2, 2);
+      Range vd = re.grown(d, 0, 1);
+      for (int m = 0; m < 3; ++m) {
+        out.cover(pi[m]);
+        in.cover(m == d ? pi[m].grown(d, 3, 2) : pi[m].grown(d, 2, 2).grown(m, 1, 0));
+        vd.cover(m == d ? pi[m].grown(d, 1, 1) : pi[m].grown(d, 0, 1).grown(m, 1, 0));
+        pi[m] = pi[m].grown(d, 2, 2);
+      }
+      b.sweep[d] = out;
+      v[d] = vd;
+      re = in;
+    }
+    for (int d = 0; d < 3; ++d) v[d].cover(pi[d]);
+  }
+  b.diffuse = b.compress = re;
+  if (diffusion)
+    for (int d = 0; d < 3; ++d) b.compress = b.compress.grown(d, 1, 1);
+  re = b.compress;
+  if (hydro) {
+    for (int d = 0; d < 3; ++d) v[d].cover(b.compress.grown(d, 0, 1));
+    b.source = v[0];
+    for (int d = 0; d < 3; ++d) {
+      b.source.cover(v[d]);
+      re.cover(v[d].grown(d, 1, 0));
+    }
+  }
+  b.before.re = re;
+  for (int d = 0; d < 3; ++d) b.before.v[d] = hydro ? v[d] : after.v[d];
+  return b;
 }
 
 template <class T>
@@ -663,6 +737,34 @@ struct Builder {
     return b;
   }
 
+  Box box(const LevelView& v, const Range& r) const {
+    Box b;
+    b.tile = 0;
+    b.zc = 0;
+    for (int d = 0; d < 3; ++d) {
+      b.lo[d] = std::max(0, r.lo[d]);
+      b.hi[d] = std::min(v.s[d], r.hi[d]);
+    }
+    b.set_divisors();
+    return b;
+  }
+
+  // What the rest of the coarse step needs of level l after its level step: the active
+  // cells.  A finer level's faces on its frontier come from its parent (CommUp); level
+  // 0's upper boundary faces are the solver's.  Where another sub-cycle follows with no
+  // CommUp in between, what that one needs.
+  StepBoxes boxes_of(const Run& r, int l, bool sub_cycle_follows) const {
+    const LevelView& v = r.L[l].v;
+    Need n;
+    for (int d = 0; d < 3; ++d) {
+      n.re.lo[d] = v.G;
+      n.re.hi[d] = v.G + v.n[d];
+    }
+    for (int d = 0; d < 3; ++d) n.v[d] = l == 0 ? n.re.grown(d, 0, 1) : n.re.grown(d, -1, 0);
+    StepBoxes b = step_boxes(n, r.P.hydro_on, r.P.chi > 0.0);
+    return sub_cycle_follows ? step_boxes(b.before, r.P.hydro_on, r.P.chi > 0.0) : b;
+  }
+
   void add(std::vector<Entry>& out, int op, int d, Item<T> it) const {
     it.b.tile = is_box_op(op) ? tiles.t[op][d] : 0;
     if (op == OP_SWEEP) it.b.zc = sweep_chunk(it.b, d);
@@ -684,8 +786,7 @@ struct Builder {
 
   void level_step(const Run& r, int l, int m_out, std::vector<Entry>& out) const {
     Item<T> it = base(r, l);
-    const bool fused_tr =
-        sweeps_fused(transport, sizeof(T) == 8 ? DF_FP64 : DF_FP32_STATE);
+    const bool fused_tr = transport != DF_TRANSPORT_SEPARATE;
     // the x sweep forms the staggered momenta from v and rho itself
     if (fused_tr) it.flags &= ~FL_WRITE_PI;
     it.b = box(it.L, m_out + kReach, r.P.av_c2 > 0.0, l == 0 ? 1 : 0);
@@ -698,6 +799,23 @@ struct Builder {
                         r.prm.xi_mode != 1 && it.L.mir == 0;
     const bool kick_done = paired && sub_of[l] == 1;
     const int vrec_d = paired && sub_of[l] == 0 ? 1 : 0;
+    // the fused sweeps' step gives each op its own box
+    const bool own_boxes = fused_tr && !full_boxes && !(r.P.av_c2 > 0.0);
+    const StepBoxes sb = boxes_of(r, l, m_out > 0);
+    if (P.hydro_on && fused_tr && !(r.P.av_c2 > 0.0)) {
+      // the velocity recovery after this step's kicks; where the first of two sub-cycles'
+      // recovery applies the second's kick, the second's
+      const Range v = boxes_of(r, l, m_out > 0 && !paired).vrec;
+      for (int d = 0; d < 3; ++d) {
+        it.again.lo[d] = std::max(0, v.lo[d]);
+        it.again.hi[d] = std::min(it.L.s[d], v.hi[d]);
+      }
+    }
+    auto boxed = [&](const Range& b) {
+      Item<T> i = it;
+      if (own_boxes) i.b = box(it.L, b);
+      return i;
+    };
     if (l == 0)
       for (int d = 0; d < 3; ++d) {
         Item<T> bc = it;
@@ -707,22 +825,23 @@ struct Builder {
       }
     else
       mirror_fill(it, out);  // CommUp filled the rest of the ghosts
-    if (P.hydro_on && !kick_done) add(out, OP_SOURCE, 0, it);
+    if (P.hydro_on && !kick_done) add(out, OP_SOURCE, 0, boxed(sb.source));
     if (P.hydro_on && P.av_c2 > 0.0) {
       add(out, OP_VISC_Q, 0, it);
       add(out, OP_VISC_V, 0, it);
     }
-    if (P.hydro_on || P.L != 0.0 || P.chi > 0.0) add(out, OP_COMPRESS, 0, it);
+    if (P.hydro_on || P.L != 0.0 || P.chi > 0.0)
+      add(out, OP_COMPRESS, 0, boxed(sb.compress));
     // before the separate transport kernels the diffusion also forms the x sweep's
     // e/rho (in Scratch::w[0]), in place of that sweep's preparation kernel
     const bool eps_x = P.chi > 0.0 && P.hydro_on && !fused_tr;
     if (P.chi > 0.0) {
       if (it.L.is_child) add(out, OP_FRONTIER_DIFF, 0, it);
-      add(out, OP_DIFFUSE, eps_x ? 1 : 0, it);
+      add(out, OP_DIFFUSE, eps_x ? 1 : 0, boxed(sb.diffuse));
     }
     if (P.hydro_on && fused_tr) {
-      for (int d = 0; d < 3; ++d) add(out, OP_SWEEP, d, it);
-      add(out, OP_VREC, vrec_d, it);
+      for (int d = 0; d < 3; ++d) add(out, OP_SWEEP, d, boxed(sb.sweep[d]));
+      add(out, OP_VREC, vrec_d, boxed(sb.vrec));
     } else if (P.hydro_on) {
       // At the x sweep the staggered momenta were just formed from v and rho (the
       // kick, or the viscosity stage after it, wrote them; nothing since has changed

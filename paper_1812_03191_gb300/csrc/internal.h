@@ -367,6 +367,16 @@ enum ItemFlags {
   FL_EPS_ONLY = 128  // TPREP: e/rho only (the x sweep reads Pi/rho_face - V from v)
 };
 
+// Where the velocity recovery of the level step stores the velocities again (nowhere by
+// default).
+struct Again {
+  int lo[3], hi[3];
+  __host__ __device__ bool has(const int c[3]) const {
+    return c[0] >= lo[0] && c[0] < hi[0] && c[1] >= lo[1] && c[1] < hi[1] && c[2] >= lo[2] &&
+           c[2] < hi[2];
+  }
+};
+
 // One work item.  Plain data, copied to shared memory by the kernel; size a
 // multiple of 16 bytes.
 template <class T>
@@ -375,6 +385,7 @@ struct __align__(16) Item {
   LevelView F;          // fine level of CommUp / CommMean
   Scratch S;            // the run's scratch
   Box b;                // box of stencil ops
+  Again again;          // the kicks: see Again
   Bg<Arith<T>> bg;
   Geo<Arith<T>> g;
   const void* dt;       // this level's step, Arith<T>

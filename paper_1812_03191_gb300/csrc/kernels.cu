@@ -139,6 +139,14 @@ __device__ __forceinline__ void st2(dstate* p, int e, df64 a, df64 b) {
   const df64 ca = canonical(a), cb = canonical(b);
   *reinterpret_cast<float4*>(p + e) = make_float4(ca.hi, ca.lo, cb.hi, cb.lo);
 }
+// A kicked velocity before the fused sweeps.  Where the level step's velocity recovery
+// stores the velocity again (`again`), the FP64 state's value stays unrounded until then,
+// so that the momenta, which the x sweep forms from it, lose nothing to the cut.
+__device__ __forceinline__ void st_kicked(float* p, int i, float v, bool) { p[i] = v; }
+__device__ __forceinline__ void st_kicked(dstate* p, int i, df64 v, bool again) {
+  const df64 c = canonical(v);
+  p[i] = again ? dstate{v.hi, v.lo} : dstate{c.hi, c.lo};
+}
 // A state value in the state's own type, for the kernels that compute in it (the
 // boundary fill, CommMean, the time step, I/O): the float itself, or the exact double
 // of a stored pair; put() stores such a value back (a double rounded to the pair).
@@ -260,7 +268,8 @@ template <class T, int NC>
 __device__ __forceinline__ void el_source(const LevelView& L, const Box& b, const Scratch& S,
                                           const Arith<T>* __restrict__ dtp, int write_pi,
                                           Arith<T> gm1, const Bg<Arith<T>>& bg,
-                                          const Geo<Arith<T>>& g, const unsigned* el) {
+                                          const Geo<Arith<T>>& g, const Again& ag,
+                                          const unsigned* el) {
   using C = Arith<T>;
   int c[NC], c3[NC][3];
   bool ok[NC];
@@ -306,7 +315,7 @@ __device__ __forceinline__ void el_source(const LevelView& L, const Box& b, cons
         C acc = mul_u(div_u(mul_u(gm1, ec[n] - em[n][d]), rf) + (fc[n] - fm[n][d]),
                       g.inv_dx[d]);
         C vn = vv[n][d] - mul_u(h, acc);
-        st((St<T>*)L.q[F_VX + d], c[n], vn);
+        st_kicked((St<T>*)L.q[F_VX + d], c[n], vn, ag.has(c3[n]));
         // momentum deviation: rf (V + dv) - rho0 V
         if (write_pi)
           st((Arith<T>*)S.pi[d], c[n], mul_u(bg.rho0, vn) + mul_u(drf, add_k(vn, bg.V[d])));
@@ -932,10 +941,13 @@ __device__ __forceinline__ void sweep_march(const Item<T>& it, int x, int row, b
   const unsigned stM = (unsigned)L.st[d] * ES;
   const unsigned c0 = (unsigned)((EDGE ? min(max(x, 0), L.s[0] - 1) : x) + row * L.st[RA]) * ES;
   const unsigned cb = EDGE && row < 1 ? c0 : c0 - (unsigned)L.st[RA] * ES;
-  const St<T>* const rhoS = (const St<T>*)(d == 1 ? it.S.F : it.S.P[0]);
-  const St<T>* const eS = (const St<T>*)(d == 1 ? it.S.E : it.S.P[1]);
-  St<T>* const rhoD = (St<T>*)(d == 1 ? it.S.P[0] : L.q[F_RHO]);
-  St<T>* const eD = (St<T>*)(d == 1 ? it.S.P[1] : L.q[F_E]);
+  // between the sweeps rho and e are unrounded (the arithmetic type); the z sweep stores
+  // the state
+  using D = std::conditional_t<d == 1, C, St<T>>;
+  const C* const rhoS = (const C*)(d == 1 ? it.S.F : it.S.P[0]);
+  const C* const eS = (const C*)(d == 1 ? it.S.E : it.S.P[1]);
+  D* const rhoD = (D*)(d == 1 ? it.S.P[0] : L.q[F_RHO]);
+  D* const eD = (D*)(d == 1 ? it.S.P[1] : L.q[F_E]);
   const St<T>* const vd = (const St<T>*)L.q[F_VX + d];
   auto piS = [&](int m) { return (const C*)(d == 1 ? it.S.pi[m] : it.S.w[m]); };
   auto piD = [&](int m) { return (C*)(d == 1 ? it.S.w[m] : it.S.pi[m]); };
@@ -1068,7 +1080,7 @@ __device__ __forceinline__ void sweep_march(const Item<T>& it, int x, int row, b
           C pv = p2[m];
           // P_d of cells r-3, r-2; the others' of planes r-2, r-1
           if (!EDGE || (upd && (m == d ? u2 >= 3 : m == 0 ? x >= 1 : row >= 1)))
-            pv = sub_u(pv, mul_u(sub_u(P[m], Pp[m]), iv));
+            pv = pv - mul_u(sub_u(P[m], Pp[m]), iv);
           stb(piD(m), c, pv);
         }
       }
@@ -1204,8 +1216,8 @@ __device__ __forceinline__ void sweep_x(const Item<T>& it, int x, int row, bool 
           rv = rv - mul_u(sub_u(Fhi, Flo), iv);
           ev = ev - mul_u(sub_u(Ehi, Elo), iv);
         }
-        stb((St<T>*)it.S.F, c, rv);
-        stb((St<T>*)it.S.E, c, ev);
+        stb((C*)it.S.F, c, rv);
+        stb((C*)it.S.E, c, ev);
 #pragma unroll
         for (int m = 0; m < 3; ++m) {
           C pv = z;  // the momentum Pi - rho0 V of v
@@ -1215,7 +1227,7 @@ __device__ __forceinline__ void sweep_x(const Item<T>& it, int x, int row, bool 
             pv = add_u(mul_u(bg.rho0, w[m]), mul_u(drf, add_k(w[m], bg.V[m])));
           }
           if (!EDGE || (upd && in && (m != 0 || x >= 3)))
-            pv = sub_u(pv, mul_u(m == 0 ? sub_u(P[0], Px_m1) : sub_u(m == 1 ? Py_p1 : Pz_p1, P[m]), iv));
+            pv = pv - mul_u(m == 0 ? sub_u(P[0], Px_m1) : sub_u(m == 1 ? Py_p1 : Pz_p1, P[m]), iv);
           stb((C*)it.S.pi[m], c, pv);
         }
       }
@@ -1261,7 +1273,8 @@ template <class T, int NC, int KICK2>
 __device__ __forceinline__ void el_vrec_source(const LevelView& L, const Box& b, const Scratch& S,
                                                const Arith<T>* __restrict__ dtp, Arith<T> gm1,
                                                const Bg<Arith<T>>& bg, const Geo<Arith<T>>& g,
-                                               int write_pi, const unsigned* el) {
+                                               const Again& ag, int write_pi,
+                                               const unsigned* el) {
   using C = Arith<T>;
   int c[NC], c3[NC][3];
   bool ok[NC];
@@ -1319,7 +1332,10 @@ __device__ __forceinline__ void el_vrec_source(const LevelView& L, const Box& b,
         if (write_pi)
           st((Arith<T>*)S.pi[d], c[n], mul_u(bg.rho0, vn) + mul_u(drf, add_k(vn, bg.V[d])));
       }
-      st((St<T>*)L.q[F_VX + d], c[n], vn);
+      if (KICK2)
+        st_kicked((St<T>*)L.q[F_VX + d], c[n], vn, ag.has(c3[n]));
+      else
+        st((St<T>*)L.q[F_VX + d], c[n], vn);
     }
   }
 }
@@ -2208,7 +2224,7 @@ __device__ __forceinline__ void run_op(const Item<T>& it, unsigned tid) {
   for (int n = 1; n < NC; ++n) el[n] = el[0] + n * kBlock;
   if (OP == OP_SOURCE)
     el_source<T, NC>(it.L, it.b, it.S, (const Arith<T>*)it.dt, it.flags & FL_WRITE_PI, it.gm1,
-                     it.bg, it.g, el);
+                     it.bg, it.g, it.again, el);
   else if (OP == OP_COMPRESS) {
     if (it.L.has_child)  // before any consumer
 #pragma unroll 1
@@ -2237,7 +2253,7 @@ __device__ __forceinline__ void run_op(const Item<T>& it, unsigned tid) {
     el_visc_v<T>(it.L, it.b, it.S, (const Arith<T>*)it.dt, it.flags & FL_WRITE_PI, it.bg, it.g, tid);
   else if (OP == OP_VREC)  // D = 1: with the next sub-cycle's first kick
     el_vrec_source<T, NC, D>(it.L, it.b, it.S, (const Arith<T>*)it.dt, it.gm1, it.bg, it.g,
-                             it.flags & FL_WRITE_PI, el);
+                             it.again, it.flags & FL_WRITE_PI, el);
   else if (OP == OP_BC)
     el_bc_axis<T>(it.L, D, it.bc_lo, it.bc_hi, (T)it.V[0], (T)it.V[1], (T)it.V[2], tid);
   else if (OP == OP_COMMUP)
