@@ -769,19 +769,26 @@ struct Builder {
     it.b.tile = is_box_op(op) ? tiles.t[op][d] : 0;
     if (op == OP_SWEEP) it.b.zc = sweep_chunk(it.b, d);
     it.br = br;
-    it.count = op_count(op, d, it.L, it.F, it.b);
+    it.count = op_count(op, d, it.L, it.F, it.b, it.bc);
     out.push_back({op, d, it});
   }
 
-  // reflect fill of the mirror sides only (type -1: the upper side is left alone)
+  // ghost fill by side types (-1: left alone), in one launch where that can be done
+  void fill(Item<T> it, const int* bc, std::vector<Entry>& out) const {
+    const bool by_axis = bc_by_axis(it.L, bc);
+    for (int d = 0; d < (by_axis ? 3 : 1); ++d) {
+      for (int k = 0; k < 6; ++k) it.bc[k] = by_axis && k / 2 != d ? -1 : bc[k];
+      add(out, OP_BC, 0, it);
+    }
+  }
+
+  // reflect fill of the mirror sides only
   void mirror_fill(const Item<T>& it, std::vector<Entry>& out) const {
-    for (int d = 0; d < 3; ++d)
-      if (it.L.mir >> d & 1) {
-        Item<T> bc = it;
-        bc.bc_lo = DF_BC_REFLECT;
-        bc.bc_hi = -1;
-        add(out, OP_BC, d, bc);
-      }
+    if (!it.L.mir) return;
+    int bc[6];
+    for (int k = 0; k < 6; ++k)
+      bc[k] = k % 2 == 0 && (it.L.mir >> (k / 2) & 1) ? DF_BC_REFLECT : -1;
+    fill(it, bc, out);
   }
 
   void level_step(const Run& r, int l, int m_out, std::vector<Entry>& out) const {
@@ -817,12 +824,7 @@ struct Builder {
       return i;
     };
     if (l == 0)
-      for (int d = 0; d < 3; ++d) {
-        Item<T> bc = it;
-        bc.bc_lo = P.bc[2 * d];
-        bc.bc_hi = P.bc[2 * d + 1];
-        add(out, OP_BC, d, bc);
-      }
+      fill(it, P.bc, out);
     else
       mirror_fill(it, out);  // CommUp filled the rest of the ghosts
     if (P.hydro_on && !kick_done) add(out, OP_SOURCE, 0, boxed(sb.source));
@@ -1058,12 +1060,7 @@ int plan_build_ops(Plan& plan, Run* r, const std::vector<std::pair<int, int>>& o
         B.add(v, op, 0, it);
         break;
       case OP_BC:
-        for (int d = 0; d < 3; ++d) {
-          Item<T> bc = it;
-          bc.bc_lo = r->P.bc[2 * d];
-          bc.bc_hi = r->P.bc[2 * d + 1];
-          B.add(v, OP_BC, d, bc);
-        }
+        B.fill(it, r->P.bc, v);
         break;
       case OP_FORCE_LEVEL:
         B.add(v, op, 0, B.force_level_item(*r, l));

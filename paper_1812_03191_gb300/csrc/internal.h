@@ -367,6 +367,54 @@ enum ItemFlags {
   FL_EPS_ONLY = 128  // TPREP: e/rho only (the x sweep reads Pi/rho_face - V from v)
 };
 
+// Ghost fill (OP_BC): the elements of the sides that are filled and, where v_d has a fixed
+// lower boundary face, that face, as six boxes: two slabs across z over the whole x-y
+// range, two across y, two across x, each within what the earlier ones left.
+__host__ __device__ inline void bc_inner(const LevelView& L, const int* bc, int* lo, int* hi) {
+  for (int d = 0; d < 3; ++d) {
+    lo[d] = bc[2 * d] < 0 ? 0 : L.G + (bc[2 * d] >= 2);
+    hi[d] = bc[2 * d + 1] < 0 ? L.s[d] : L.G + L.n[d];
+  }
+}
+__host__ __device__ inline long long bc_elements(const LevelView& L, const int* bc) {
+  int lo[3], hi[3];
+  bc_inner(L, bc, lo, hi);
+  return (long long)L.s[0] * L.s[1] * L.s[2] -
+         (long long)(hi[0] - lo[0]) * (hi[1] - lo[1]) * (hi[2] - lo[2]);
+}
+// does the lower wall of axis d mirror the upper boundary face, which is filled too?
+__host__ __device__ inline bool bc_wraps(const LevelView& L, const int* bc, int d) {
+  return L.n[d] == L.G && bc[2 * d] == 3 && (bc[2 * d + 1] == 0 || bc[2 * d + 1] >= 2);
+}
+__host__ __device__ inline bool bc_by_axis(const LevelView& L, const int* bc) {
+  return bc_wraps(L, bc, 0) || bc_wraps(L, bc, 1) || bc_wraps(L, bc, 2);
+}
+// the t-th of them; false past the last
+__host__ __device__ inline bool bc_element(const LevelView& L, const int* bc, unsigned t,
+                                           int* c) {
+  int in_lo[3], in_hi[3], lo[3] = {0, 0, 0}, hi[3] = {L.s[0], L.s[1], L.s[2]};
+  bc_inner(L, bc, in_lo, in_hi);
+  for (int d = 2; d >= 0; --d) {
+    for (int side = 0; side < 2; ++side) {
+      const int l = side ? in_hi[d] : 0, e = side ? L.s[d] - in_hi[d] : in_lo[d];
+      unsigned w[3];
+      for (int k = 0; k < 3; ++k) w[k] = (unsigned)(k == d ? e : hi[k] - lo[k]);
+      const unsigned n = w[0] * w[1] * w[2];
+      if (t < n) {
+        const unsigned q = t / w[0], z = q / w[1];
+        c[0] = (d == 0 ? l : lo[0]) + (int)(t - q * w[0]);
+        c[1] = (d == 1 ? l : lo[1]) + (int)(q - z * w[1]);
+        c[2] = (d == 2 ? l : lo[2]) + (int)z;
+        return true;
+      }
+      t -= n;
+    }
+    lo[d] = in_lo[d];
+    hi[d] = in_hi[d];
+  }
+  return false;
+}
+
 // Where the velocity recovery of the level step stores the velocities again (nowhere by
 // default).
 struct Again {
@@ -398,7 +446,8 @@ struct __align__(16) Item {
   Arith<T> gm1, lum, av;
   Arith<T> gga;         // gamma (gamma - 1), the time step's per-cell factor
   double gg, rho0d, e0d, V[3], dt_fixed;
-  int ring_cap, npart, level, band, flags, bc_lo, bc_hi;
+  int ring_cap, npart, level, band, flags;
+  int bc[6];            // OP_BC: type of every side, -1 to leave it alone
   unsigned count;       // index-space size of the item
   unsigned br;          // bit m: inside the second sub-cycle of level m + 1 (skipped
                         // when the search chose xi_m = 1)
@@ -430,7 +479,8 @@ template <class T>
 int launch_batch(int op, int d, const Item<T>* items, const unsigned* starts, int nitems,
                  unsigned nchunks, unsigned grid, cudaStream_t st, const Item<T>* host_item);
 int op_chunk_elems(int op, int esz);  // elements per chunk for state elements of esz bytes
-unsigned op_count(int op, int d, const LevelView& L, const LevelView& F, const Box& b);
+unsigned op_count(int op, int d, const LevelView& L, const LevelView& F, const Box& b,
+                  const int* bc);
 int force_partials_per_level(const LevelView& L);
 int launch_force_weights(const LevelView& L, const Phys& P, cudaStream_t st);
 template <class T> int launch_init_uniform(const LevelView& L, const Phys& P, cudaStream_t st);
