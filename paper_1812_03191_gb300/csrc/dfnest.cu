@@ -892,36 +892,52 @@ struct Builder {
     }
   }
 
-  Item<T> force_level_item(const Run& r, int l) const {
-    Item<T> f = base(r, l);
-    int off = 0;
-    for (int m = 0; m < l; ++m) off += force_partials_per_level(r.L[m].v);
-    f.partials = r.partials + 3 * off;
-    return f;
+  // a reduction over every level of a run: its chunks in all
+  unsigned chunks_of(const Run& r, int op) const {
+    const unsigned ce = (unsigned)op_chunk_elems(op, (int)sizeof(T));
+    unsigned n = 0;
+    for (int l = 0; l < r.nl; ++l) {
+      const Item<T> it = base(r, l);
+      n += (op_count(op, 0, it.L, it.F, it.b, it.bc) + ce - 1) / ce;
+    }
+    return n;
   }
 
-  Item<T> force_final_item(const Run& r, bool ring) const {
-    Item<T> ff = base(r, 0);
-    ff.partials = r.partials;
-    ff.npart = r.n_partials;
-    if (ring) {
-      ff.ring = r.ring;
-      ff.ring_pos = r.ring_pos;
-      ff.ring_cap = r.ring_cap;
+  // the time step (Eq. 55) of a run
+  void add_dt(const Run& r, int ri, std::vector<Entry>& out) const {
+    for (int l = 0; l < r.nl; ++l) {
+      Item<T> it = base(r, l);
+      it.fin = d_fins + ri;
+      it.n_levels = r.nl;
+      it.total = chunks_of(r, OP_DT_LEVEL);
+      add(out, OP_DT_LEVEL, 0, it);
     }
-    return ff;
+  }
+
+  // the force (Eq. 18) of a run; with `ring`, as the end of a coarse step: into the force
+  // history, and the time advances
+  void add_force(const Run& r, bool ring, std::vector<Entry>& out) const {
+    int off = 0;
+    for (int l = 0; l < r.nl; ++l) {
+      Item<T> it = base(r, l);
+      it.partials = r.partials + 3 * off;
+      off += force_partials_per_level(r.L[l].v);
+      it.run_partials = r.partials;
+      it.npart = r.n_partials;
+      it.total = chunks_of(r, OP_FORCE_LEVEL);
+      if (ring) {
+        it.ring = r.ring;
+        it.ring_pos = r.ring_pos;
+        it.ring_cap = r.ring_cap;
+      }
+      add(out, OP_FORCE_LEVEL, 0, it);
+    }
   }
 
   void coarse_step(const Run& r, int ri, std::vector<Entry>& out) const {
-    for (int l = 0; l < r.nl; ++l) add(out, OP_DT_LEVEL, 0, base(r, l));
-    Item<T> fin = base(r, 0);
-    fin.level = r.nl;  // the finalisation covers all levels
-    fin.fin = d_fins + ri;
-    add(out, OP_DT_FINAL, 0, fin);
+    add_dt(r, ri, out);
     advance(r, 0, 0, out);
-    for (int l = 0; l < r.nl; ++l) add(out, OP_FORCE_LEVEL, 0, force_level_item(r, l));
-    add(out, OP_FORCE_FINAL, 0, force_final_item(r, true));
-    add(out, OP_TIME, 0, base(r, 0));
+    add_force(r, true, out);
   }
 
   // greedy merge: repeatedly launch the op kind that heads the most runs' lists,
@@ -955,17 +971,20 @@ struct Builder {
       unsigned chunks = 0;
       unsigned ce = (unsigned)op_chunk_elems(L.op, (int)sizeof(T));
       for (size_t r = 0; r < nr; ++r) {
-        if (pos[r] >= per_run[r].size()) continue;
-        const Entry& e = per_run[r][pos[r]];
-        if (e.op != best.first || e.d != best.second) continue;
-        ++pos[r];
-        unsigned nch = (e.it.count + ce - 1) / ce;
-        if (nch == 0) continue;
-        const unsigned char* p = reinterpret_cast<const unsigned char*>(&e.it);
-        plan.items.insert(plan.items.end(), p, p + sizeof(Item<T>));
-        plan.starts.push_back(chunks);
-        chunks += nch;
-        ++L.nitems;
+        while (pos[r] < per_run[r].size()) {
+          const Entry& e = per_run[r][pos[r]];
+          if (e.op != best.first || e.d != best.second) break;
+          ++pos[r];
+          unsigned nch = (e.it.count + ce - 1) / ce;
+          if (nch) {
+            const unsigned char* p = reinterpret_cast<const unsigned char*>(&e.it);
+            plan.items.insert(plan.items.end(), p, p + sizeof(Item<T>));
+            plan.starts.push_back(chunks);
+            chunks += nch;
+            ++L.nitems;
+          }
+          if (!is_joined_op(e.op)) break;
+        }
       }
       L.nchunks = chunks;
       if (L.nitems) plan.launches.push_back(L);
@@ -1047,8 +1066,7 @@ int plan_build_ops(Plan& plan, Run* r, const std::vector<std::pair<int, int>>& o
   for (auto& ol : ops) {
     int op = ol.first, l = ol.second;
     Item<T> it = B.base(*r, l);
-    // box ops over the whole array; the reductions keep base()'s active box
-    if (op != OP_DT_LEVEL && op != OP_FORCE_LEVEL) it.b = B.box(it.L, it.L.G);
+    it.b = B.box(it.L, it.L.G);  // the whole array
     switch (op) {
       case OP_COMMUP:
         B.mirror_fill(it, v);  // as in the coarse step: the stencil reaches across a plane
@@ -1062,16 +1080,11 @@ int plan_build_ops(Plan& plan, Run* r, const std::vector<std::pair<int, int>>& o
       case OP_BC:
         B.fill(it, r->P.bc, v);
         break;
-      case OP_FORCE_LEVEL:
-        B.add(v, op, 0, B.force_level_item(*r, l));
+      case OP_FORCE_LEVEL:  // of every level
+        B.add_force(*r, false, v);
         break;
-      case OP_FORCE_FINAL:
-        B.add(v, op, 0, B.force_final_item(*r, false));
-        break;
-      case OP_DT_FINAL:
-        it.level = r->nl;
-        it.fin = plan.d_fins;
-        B.add(v, op, 0, it);
+      case OP_DT_LEVEL:
+        B.add_dt(*r, 0, v);
         break;
       default:
         B.add(v, op, 0, it);
@@ -1624,10 +1637,7 @@ int df_force_now(df_ctx* c, double F[3]) {
   if (!F) return fail(DF_EINVAL, "null output");
   DevGuard g(c->device);
   enter(c);
-  std::vector<std::pair<int, int>> ops;
-  for (int l = 0; l < c->run->nl; ++l) ops.push_back({OP_FORCE_LEVEL, l});
-  ops.push_back({OP_FORCE_FINAL, 0});
-  int rc = run_ops_now(c->run, c->x, ops);
+  int rc = run_ops_now(c->run, c->x, {{OP_FORCE_LEVEL, 0}});
   leave(c);
   if (rc) return rc;
   DevScalars h;
@@ -1668,10 +1678,7 @@ int df_compute_dt(df_ctx* c, double* dt, double* dt_level) {
   DevScalars before;
   CK(cudaMemcpyAsync(&before, r->ds, sizeof before, cudaMemcpyDeviceToHost, c->x.st));
   CK(cudaStreamSynchronize(c->x.st));
-  std::vector<std::pair<int, int>> ops;
-  for (int l = 0; l < r->nl; ++l) ops.push_back({OP_DT_LEVEL, l});
-  ops.push_back({OP_DT_FINAL, 0});
-  int rc = run_ops_now(r, c->x, ops);
+  int rc = run_ops_now(r, c->x, {{OP_DT_LEVEL, 0}});
   if (rc) return rc;
   DevScalars after;
   CK(cudaMemcpy(&after, r->ds, sizeof after, cudaMemcpyDeviceToHost));

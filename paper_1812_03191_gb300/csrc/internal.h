@@ -178,6 +178,7 @@ struct DevScalars {
   df64 kd[16][12];
   float kf[16][12];
   int unhealthy;
+  unsigned dt_done, force_done;  // chunks of the running reductions that are through
   unsigned xi1;  // bit m set when the Eq. 55-56 search chose xi_m = 1 this coarse step
 };
 
@@ -271,14 +272,20 @@ struct DtFinal {
 // Ops of the work-list kernel.  Every launch runs one op over a list of work
 // items; an item is one (run, level) with its box and its own parameters.
 // OP_TFRONTIER and OP_ZERO_ACC are no longer emitted (the CommFlux record replaced
-// them); they keep their numbers so that op indices (tile-shape controls, timing
-// kinds, the binding's op names) stay stable.
+// them), nor are OP_DT_FINAL, OP_FORCE_FINAL and OP_TIME (the last chunk of OP_DT_LEVEL and
+// OP_FORCE_LEVEL does their work); they keep their numbers so that op indices (tile-shape
+// controls, timing kinds, the binding's op names) stay stable.
 enum Op {
   OP_SOURCE = 0, OP_COMPRESS, OP_FRONTIER_DIFF, OP_DIFFUSE, OP_TPREP, OP_TFLUX, OP_TFRONTIER,
   OP_TMOM, OP_TUPDATE, OP_VREC, OP_BC, OP_COMMUP, OP_COMMMEAN, OP_ZERO_ACC, OP_DT_LEVEL,
   OP_DT_FINAL, OP_FORCE_LEVEL, OP_FORCE_FINAL, OP_TIME, OP_SWEEP, OP_VISC_Q, OP_VISC_V,
   OP_COUNT
 };
+
+// ops whose consecutive items of one run are independent and share a launch
+__host__ __device__ constexpr bool is_joined_op(int op) {
+  return op == OP_DT_LEVEL || op == OP_FORCE_LEVEL;
+}
 
 // ops that enumerate the elements of a box (the ones a tile shape applies to)
 __host__ __device__ inline bool is_box_op(int op) {
@@ -439,8 +446,9 @@ struct __align__(16) Item {
   const void* dt;       // this level's step, Arith<T>
   const void* kc;       // this level step's constants (DevScalars::kd / kf), Arith<T>
   DevScalars* ds;       // the run's scalars
-  const DtFinal* fin;   // OP_DT_FINAL constants
-  double* partials;     // force partials (this level's first, or the run's for the final sum)
+  const DtFinal* fin;   // the time step's constants
+  double* partials;     // force partials of this level
+  const double* run_partials;  // and of the run, for the final sum
   double* ring;         // force history
   long long* ring_pos;
   Arith<T> gm1, lum, av;
@@ -448,6 +456,8 @@ struct __align__(16) Item {
   double gg, rho0d, e0d, V[3], dt_fixed;
   int ring_cap, npart, level, band, flags;
   int bc[6];            // OP_BC: type of every side, -1 to leave it alone
+  int n_levels;         // reductions: the run's levels and their chunks in all
+  unsigned total;
   unsigned count;       // index-space size of the item
   unsigned br;          // bit m: inside the second sub-cycle of level m + 1 (skipped
                         // when the search chose xi_m = 1)

@@ -1635,6 +1635,27 @@ __device__ __forceinline__ void el_commmean(const LevelView& C, const LevelView&
   }
 }
 
+// ------------------------------------------------------------ reductions of a run
+// True in the last of a run's `total` chunks of one reduction to get here: every chunk's
+// results are then visible (read them past L1).  Each chunk counts itself after its
+// results are written; the last one clears the count for the next step.  Nothing waits.
+// The final step of a reduction then needs no launch of its own, and the levels share one
+// (one 32^3 level: 13 launches, 67.7 us a coarse step -> 10, 66.2; 3 x 64^3 FP64 69, 834
+// us -> 62, 800; 16 serving runs 99, 874 us -> 71, 770).
+__device__ __forceinline__ bool last_chunk(unsigned* done, unsigned total) {
+  __shared__ int s_last;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    const bool last = atomicAdd(done, 1u) == total - 1u;
+    if (last) *done = 0u;
+    __threadfence();
+    s_last = last;
+  }
+  __syncthreads();
+  return s_last != 0;
+}
+
 // ------------------------------------------------------------- time step
 __device__ __forceinline__ float warp_max_t(float v) {
 #pragma unroll
@@ -1756,7 +1777,7 @@ __device__ __forceinline__ void el_dt_level(const LevelView& L, const Box& b, in
         const A cs = dsqrt(hdiv(gga * ee, r));
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
-          const A v0 = dabs(bg.V[d] + va[u][d]), v1 = dabs(bg.V[d] + vb[u][d]);
+          const A v0 = dabs(add_k(va[u][d], bg.V[d])), v1 = dabs(add_k(vb[u][d], bg.V[d]));
           mx[d] = dmax(mx[d], cs + dmax(v0, v1));
         }
       }
@@ -1783,27 +1804,29 @@ __device__ __forceinline__ void el_dt_level(const LevelView& L, const Box& b, in
   }
 }
 
-// Eq. 55: dt = min_l dt_l prod_{m<l} xi_m; resets the per-level maxima
+// Eq. 55: dt = min_l dt_l prod_{m<l} xi_m; resets the per-level maxima.  One block; a
+// thread per level and axis, then per level, per sub-cycling word and per constant.
 __device__ __forceinline__ void el_dt_finalize(DevScalars* ds, int n_levels, const DtFinal& fin,
                                                double dt_fixed) {
-  __shared__ double s_lim[16];
+  __shared__ double s_adv[48], s_lim[16], s_prod[16], s_dt;
   __shared__ double s_ratio[kBlock];
   __shared__ int s_word[kBlock];
-  if (threadIdx.x == 0) {
-    for (int l = 0; l < n_levels; ++l) {
-      double lim = fin.diff_lim[l];
-      for (int d = 0; d < 3; ++d) {
-        double mx = __longlong_as_double((long long)ds->dtmin[3 * l + d]);
-        double t = fin.cfl_dx[l][d] / mx;  // +inf when the maximum is 0
-        if (t < lim) lim = t;
-        ds->dtmin[3 * l + d] = 0ull;
-      }
-      ds->dtlev[l] = lim;
-      s_lim[l] = lim;
-    }
+  const int t = threadIdx.x;
+  if (t < 3 * n_levels) {
+    const double mx = __longlong_as_double((long long)__ldcg(&ds->dtmin[t]));
+    s_adv[t] = fin.cfl_dx[t / 3][t % 3] / mx;  // +inf when the maximum is 0
+    ds->dtmin[t] = 0ull;
   }
   __syncthreads();
-  double prod[16];
+  if (t < n_levels) {
+    double lim = fin.diff_lim[t];
+    for (int d = 0; d < 3; ++d)
+      if (s_adv[3 * t + d] < lim) lim = s_adv[3 * t + d];
+    ds->dtlev[t] = lim;
+    s_lim[t] = lim;
+    s_prod[t] = fin.prod[t];
+  }
+  __syncthreads();
   unsigned xi1 = 0;
   if (fin.search && n_levels > 1) {
     // Eq. 55-56: the word xi_m in {1, 2} (bit m of w set: xi_m = 2) with the largest
@@ -1812,12 +1835,12 @@ __device__ __forceinline__ void el_dt_finalize(DevScalars* ds, int n_levels, con
     const int nw = n_levels - 1;
     double best = -1.0;
     int bw = 0;
-    for (int w = threadIdx.x; w < (1 << nw); w += kBlock) {
+    for (int w = t; w < (1 << nw); w += kBlock) {
       double dt = INFINITY, C = 0.0, pr = 1.0;
       for (int l = 0; l < n_levels; ++l) {
         if (l > 0) pr *= ((w >> (l - 1)) & 1) ? 2.0 : 1.0;
-        const double t = s_lim[l] * pr;
-        if (t < dt) dt = t;
+        const double tl = s_lim[l] * pr;
+        if (tl < dt) dt = tl;
         C += fin.cost[l] * pr;
       }
       const double ratio = dt / C;
@@ -1826,16 +1849,16 @@ __device__ __forceinline__ void el_dt_finalize(DevScalars* ds, int n_levels, con
         bw = w;
       }
     }
-    s_ratio[threadIdx.x] = best;
-    s_word[threadIdx.x] = bw;
+    s_ratio[t] = best;
+    s_word[t] = bw;
     __syncthreads();
     for (int h = kBlock / 2; h > 0; h >>= 1) {
-      if ((int)threadIdx.x < h) {
-        const double r2 = s_ratio[threadIdx.x + h];
-        const int w2 = s_word[threadIdx.x + h];
-        if (r2 > s_ratio[threadIdx.x] || (r2 == s_ratio[threadIdx.x] && w2 < s_word[threadIdx.x])) {
-          s_ratio[threadIdx.x] = r2;
-          s_word[threadIdx.x] = w2;
+      if (t < h) {
+        const double r2 = s_ratio[t + h];
+        const int w2 = s_word[t + h];
+        if (r2 > s_ratio[t] || (r2 == s_ratio[t] && w2 < s_word[t])) {
+          s_ratio[t] = r2;
+          s_word[t] = w2;
         }
       }
       __syncthreads();
@@ -1848,37 +1871,36 @@ __device__ __forceinline__ void el_dt_finalize(DevScalars* ds, int n_levels, con
         pr *= two ? 2.0 : 1.0;
         if (!two) xi1 |= 1u << (l - 1);
       }
-      prod[l] = pr;
-    }
-  } else {
-    for (int l = 0; l < n_levels; ++l) prod[l] = fin.prod[l];
-  }
-  if (threadIdx.x != 0) return;
-  double dt = INFINITY;
-  for (int l = 0; l < n_levels; ++l) {
-    double t = s_lim[l] * prod[l];
-    if (t < dt) dt = t;
-  }
-  if (dt_fixed > 0.0) dt = dt_fixed;
-  ds->dt = dt;
-  ds->xi1 = xi1;
-  // level steps take dt / prod_{m<l} xi_m (a power of two: exact)
-  for (int l = 0; l < n_levels; ++l) {
-    double dl = dt / prod[l];
-    ds->dtl[l] = dl;
-    ds->dtf[l] = (float)dl;
-    ds->dtd[l] = to_df64(dl);
-    // the level step's constants, once here instead of in every thread
-    for (int q = 0; q < 12; ++q) {
-      const double k = fin.kfac[l][q] * dl;
-      ds->kd[l][q] = to_df64(k);
-      ds->kf[l][q] = (float)k;
+      if (t == 0) s_prod[l] = pr;
     }
   }
-}
-
-__device__ __forceinline__ void el_time_advance(DevScalars* ds) {
-  if (threadIdx.x == 0) ds->t += ds->dt;
+  if (t == 0) {
+    double dt = INFINITY;
+    for (int l = 0; l < n_levels; ++l) {
+      const double tl = s_lim[l] * s_prod[l];
+      if (tl < dt) dt = tl;
+    }
+    if (dt_fixed > 0.0) dt = dt_fixed;
+    s_dt = dt;
+    ds->dt = dt;
+    ds->xi1 = xi1;
+  }
+  __syncthreads();
+  // level steps take dt / prod_{m<l} xi_m (a power of two: exact), and their constants
+  // are formed once here instead of in every thread of the level step
+  for (int i = t; i < 13 * n_levels; i += kBlock) {
+    const int l = i / 13, q = i - 13 * l;
+    const double dl = s_dt / s_prod[l];
+    if (q == 12) {
+      ds->dtl[l] = dl;
+      ds->dtf[l] = (float)dl;
+      ds->dtd[l] = to_df64(dl);
+    } else {
+      const double c = fin.kfac[l][q] * dl;
+      ds->kd[l][q] = to_df64(c);
+      ds->kf[l][q] = (float)c;
+    }
+  }
 }
 
 // ------------------------------------------------------------------ force
@@ -1950,22 +1972,30 @@ __global__ void __launch_bounds__(kBlock) k_force_weights(LevelView L, double GM
   fw[t + 2 * na] = L.mir & 4 ? 0.0 : mult * (w * z);
 }
 
+constexpr int kPartialsAhead = 8;
 // fixed-order compensated (Neumaier) sum of the block partials, one warp per
 // component (threads 96.. of the block only take part in the barrier)
-__device__ __forceinline__ void el_force_finalize(const double* __restrict__ partials, int n,
+__device__ __forceinline__ void el_force_finalize(const double* partials, int n,
                                                   DevScalars* ds, double* ring, int ring_cap,
                                                   long long* ring_pos) {
   int comp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (comp < 3) {
     double s = 0.0, cmp = 0.0;
-    for (int p = lane; p < n; p += 32) {
-      double v = partials[3 * p + comp];
-      double tt = s + v;
-      if (fabs(s) >= fabs(v))
-        cmp += (s - tt) + v;
-      else
-        cmp += (v - tt) + s;
-      s = tt;
+    for (int p = lane; p < n; p += 32 * kPartialsAhead) {
+      double v[kPartialsAhead];  // that many in flight, added in order
+#pragma unroll
+      for (int k = 0; k < kPartialsAhead; ++k)
+        v[k] = p + 32 * k < n ? __ldcg(&partials[3 * (p + 32 * k) + comp]) : 0.0;
+#pragma unroll
+      for (int k = 0; k < kPartialsAhead; ++k) {
+        if (p + 32 * k >= n) break;
+        const double tt = s + v[k];
+        if (fabs(s) >= fabs(v[k]))
+          cmp += (s - tt) + v[k];
+        else
+          cmp += (v[k] - tt) + s;
+        s = tt;
+      }
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -1989,8 +2019,9 @@ __device__ __forceinline__ void el_force_finalize(const double* __restrict__ par
   }
   __syncthreads();
   if (threadIdx.x == 0 && ring) {
-    // the time at the end of this coarse step (the time update follows this op)
-    ring[kRingStride * (*ring_pos % ring_cap) + 3] = ds->t + ds->dt;
+    // the end of this coarse step
+    ds->t += ds->dt;
+    ring[kRingStride * (*ring_pos % ring_cap) + 3] = ds->t;
     *ring_pos += 1;
   }
 }
@@ -2266,17 +2297,16 @@ __device__ __forceinline__ void run_op(const Item<T>& it, unsigned tid) {
     el_commup<T>(it.L, it.F, tid);
   else if (OP == OP_COMMMEAN)
     el_commmean<T>(it.L, it.F, it.band, tid);
-  else if (OP == OP_DT_LEVEL)
+  else if (OP == OP_DT_LEVEL) {
     el_dt_level<T>(it.L, it.b, it.level, it.gg, it.gga, it.flags & FL_HYDRO, it.ds, it.rho0d, it.e0d,
                    it.V[0], it.V[1], it.V[2], it.bg, tid);
-  else if (OP == OP_DT_FINAL)
-    el_dt_finalize(it.ds, it.level, *it.fin, it.dt_fixed);
-  else if (OP == OP_FORCE_LEVEL)
+    if (last_chunk(&it.ds->dt_done, it.total))
+      el_dt_finalize(it.ds, it.n_levels, *it.fin, it.dt_fixed);
+  } else if (OP == OP_FORCE_LEVEL) {
     el_force_level<T>(it.L, it.b, it.L.fw, it.partials, tid);
-  else if (OP == OP_FORCE_FINAL)
-    el_force_finalize(it.partials, it.npart, it.ds, it.ring, it.ring_cap, it.ring_pos);
-  else if (OP == OP_TIME)
-    el_time_advance(it.ds);
+    if (last_chunk(&it.ds->force_done, it.total))
+      el_force_finalize(it.run_partials, it.npart, it.ds, it.ring, it.ring_cap, it.ring_pos);
+  }
 }
 
 // Persistent work-list kernel: block b takes the contiguous chunks
@@ -2334,6 +2364,27 @@ template <class T, int OP, int D>
 __global__ void __launch_bounds__(kBlock) k_single(const Item<T> it) {
   pdl_enter();
   run_op<T, OP, D>(it, blockIdx.x * kBlock + threadIdx.x);
+  pdl_exit();
+}
+
+// Reduction over several items (a run's levels, or those of many runs): one block per
+// chunk, the item read in place.  The persistent form above, with its staged item, a
+// private copy and a barrier per chunk, ran the FP64 time step of 5 x 128^3 in 413 us
+// against 222.  Three blocks an SM (80 registers): with two, 275 us.
+template <class T, int OP>
+__global__ void __launch_bounds__(kBlock, 3) k_reduce(const Item<T>* __restrict__ items,
+                                                   const unsigned* __restrict__ starts,
+                                                   int nitems) {
+  pdl_enter();
+  int lo = 0, hi = nitems - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (starts[mid] <= blockIdx.x)
+      lo = mid;
+    else
+      hi = mid - 1;
+  }
+  run_op<T, OP, 0>(items[lo], (blockIdx.x - starts[lo]) * kBlock + threadIdx.x);
   pdl_exit();
 }
 
@@ -2417,6 +2468,8 @@ static void launch_one(const Item<T>* items, const unsigned* starts, int nitems,
                        unsigned grid, cudaStream_t st, const Item<T>* host_item) {
   if (nitems == 1 && host_item)
     launch_pdl(k_single<T, OP, D>, nchunks, kBlock, st, *host_item);
+  else if constexpr (is_joined_op(OP))
+    launch_pdl(k_reduce<T, OP>, nchunks, kBlock, st, items, starts, nitems);
   else
     launch_pdl(k_batch<T, OP, D>, grid, kBlock, st, items, starts, nitems, nchunks);
 }
@@ -2456,10 +2509,7 @@ int launch_batch(int op, int d, const Item<T>* items, const unsigned* starts, in
     DFN_OP(OP_COMMUP)
     DFN_OP(OP_COMMMEAN)
     DFN_OP(OP_DT_LEVEL)
-    DFN_OP(OP_DT_FINAL)
     DFN_OP(OP_FORCE_LEVEL)
-    DFN_OP(OP_FORCE_FINAL)
-    DFN_OP(OP_TIME)
     DFN_OP(OP_VISC_Q)
     DFN_OP(OP_VISC_V)
     case OP_SWEEP:
