@@ -770,6 +770,13 @@ struct Builder {
     if (op == OP_SWEEP) it.b.zc = sweep_chunk(it.b, d);
     it.br = br;
     it.count = op_count(op, d, it.L, it.F, it.b, it.bc);
+    if (op == OP_DIFFUSE) {
+      // then the chunks that write a child's frontier record: a thread per fine face
+      const unsigned ce = (unsigned)op_chunk_elems(op, (int)sizeof(T));
+      it.box_chunks = (it.count + ce - 1) / ce;
+      const unsigned faces = it.L.is_child ? 24u * (unsigned)it.L.acc_slots : 0u;
+      it.count = (it.box_chunks + (faces + kBlockThreads - 1) / kBlockThreads) * ce;
+    }
     out.push_back({op, d, it});
   }
 
@@ -838,7 +845,6 @@ struct Builder {
     // e/rho (in Scratch::w[0]), in place of that sweep's preparation kernel
     const bool eps_x = P.chi > 0.0 && P.hydro_on && !fused_tr;
     if (P.chi > 0.0) {
-      if (it.L.is_child) add(out, OP_FRONTIER_DIFF, 0, it);
       add(out, OP_DIFFUSE, eps_x ? 1 : 0, boxed(sb.diffuse));
     }
     if (P.hydro_on && fused_tr) {

@@ -86,6 +86,7 @@ struct Box {
   }
 };
 
+constexpr int kBlockThreads = 256;  // of every kernel but the sweeps
 constexpr int kNumTiles = 5;
 // tile extents (x, y, z) with x*y*z = 256 of shape k (k = 0: flat enumeration)
 __host__ __device__ inline int tile_extent(int k, int axis) {
@@ -273,7 +274,7 @@ struct DtFinal {
 // items; an item is one (run, level) with its box and its own parameters.
 // OP_TFRONTIER and OP_ZERO_ACC are no longer emitted (the CommFlux record replaced
 // them), nor are OP_DT_FINAL, OP_FORCE_FINAL and OP_TIME (the last chunk of OP_DT_LEVEL and
-// OP_FORCE_LEVEL does their work); they keep their numbers so that op indices (tile-shape
+// OP_FORCE_LEVEL does their work), nor OP_FRONTIER_DIFF (chunks of OP_DIFFUSE); they keep their numbers so that op indices (tile-shape
 // controls, timing kinds, the binding's op names) stay stable.
 enum Op {
   OP_SOURCE = 0, OP_COMPRESS, OP_FRONTIER_DIFF, OP_DIFFUSE, OP_TPREP, OP_TFLUX, OP_TFRONTIER,
@@ -458,6 +459,7 @@ struct __align__(16) Item {
   int bc[6];            // OP_BC: type of every side, -1 to leave it alone
   int n_levels;         // reductions: the run's levels and their chunks in all
   unsigned total;
+  unsigned box_chunks;  // diffusion: chunks of the box; the rest write the frontier record
   unsigned count;       // index-space size of the item
   unsigned br;          // bit m: inside the second sub-cycle of level m + 1 (skipped
                         // when the search chose xi_m = 1)

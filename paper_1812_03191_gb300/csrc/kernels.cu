@@ -25,7 +25,7 @@ namespace dfn {
 
 namespace {
 
-constexpr int kBlock = 256;
+constexpr int kBlock = kBlockThreads;
 
 // box element t -> (i, j, k); boxes hold fewer than 2^31 elements
 __device__ __forceinline__ bool decode(const Box& b, unsigned t, int& i, int& j, int& k) {
@@ -586,9 +586,9 @@ __device__ __forceinline__ void el_diffuse(const LevelView& L, const Box& b, con
   }
 }
 
-// CommFlux record of the diffusive energy fluxes through a child's frontier faces:
-// one thread per fine frontier face (a launch of its own:
-// inside the diffusion kernel the record code would cost that kernel occupancy)
+// CommFlux record of the diffusive energy fluxes through a child's frontier faces: one
+// thread per fine frontier face, in chunks of the diffusion's launch of their own (both
+// only read rho and e/rho; as a launch it took 1.5-3 us per child level step)
 template <class T>
 __device__ __forceinline__ void el_frontier_diff(const LevelView& L, const Scratch& S,
                                                  const Arith<T>* __restrict__ kc,
@@ -2249,6 +2249,17 @@ __device__ __forceinline__ bool skipped(const Item<T>& it) {
   return it.br != 0u && (it.br & it.ds->xi1) != 0u;
 }
 
+// The chunks of the diffusion that write the frontier record: past the box's.  True if
+// this was one.
+template <class T, int OP>
+__device__ __forceinline__ bool run_record(const Item<T>& it, unsigned chunk) {
+  if (OP != OP_DIFFUSE || chunk < it.box_chunks) return false;
+  if (!skipped(it))
+    el_frontier_diff<T>(it.L, it.S, (const Arith<T>*)it.kc, it.bg.rho0, it.flags & FL_DFR, it.sub,
+                        (chunk - it.box_chunks) * kBlock + threadIdx.x);
+  return true;
+}
+
 template <class T, int OP, int D>
 __device__ __forceinline__ void run_op(const Item<T>& it, unsigned tid) {
   if (skipped(it)) return;
@@ -2270,9 +2281,6 @@ __device__ __forceinline__ void run_op(const Item<T>& it, unsigned tid) {
                            it.flags & FL_SS3, it.flags & FL_LUM, it.flags & FL_EPS, it.bg, it.g,
                            el);
   }
-  else if (OP == OP_FRONTIER_DIFF)
-    el_frontier_diff<T>(it.L, it.S, (const Arith<T>*)it.kc, it.bg.rho0, it.flags & FL_DFR, it.sub,
-                        tid);
   else if (OP == OP_DIFFUSE)  // D = 1: with the x sweep's preparation
     el_diffuse<T, NC, D>(it.L, it.b, it.S, (const Arith<T>*)it.kc, it.bg.rho0, it.flags & FL_DFR,
                          it.g, it.bg, el);
@@ -2347,8 +2355,9 @@ __global__ void __launch_bounds__(kBlock, cells_per_thread(OP, (int)sizeof(T)) =
     // fields the op uses stay in registers); ops that index the item's arrays with
     // run-time indices read it from shared memory instead
     constexpr bool kLocal =
-        !(OP == OP_COMPRESS || OP == OP_FRONTIER_DIFF || OP == OP_BC || OP == OP_COMMUP);
-    if (kLocal) {
+        !(OP == OP_COMPRESS || OP == OP_BC || OP == OP_COMMUP);
+    if (run_record<T, OP>(it, ch - starts[cur])) {
+    } else if (kLocal) {
       const Item<T> loc = it;
       run_op<T, OP, D>(loc, (ch - starts[cur]) * kBlock + threadIdx.x);
     } else {
@@ -2363,7 +2372,8 @@ __global__ void __launch_bounds__(kBlock, cells_per_thread(OP, (int)sizeof(T)) =
 template <class T, int OP, int D>
 __global__ void __launch_bounds__(kBlock) k_single(const Item<T> it) {
   pdl_enter();
-  run_op<T, OP, D>(it, blockIdx.x * kBlock + threadIdx.x);
+  if (!run_record<T, OP>(it, blockIdx.x))
+    run_op<T, OP, D>(it, blockIdx.x * kBlock + threadIdx.x);
   pdl_exit();
 }
 
@@ -2492,7 +2502,6 @@ int launch_batch(int op, int d, const Item<T>* items, const unsigned* starts, in
   switch (op) {
     DFN_OP(OP_SOURCE)
     DFN_OP(OP_COMPRESS)
-    DFN_OP(OP_FRONTIER_DIFF)
     case OP_DIFFUSE:  // d = 1: with the x sweep's preparation
       if (d == 0) launch_one<T, OP_DIFFUSE, 0>(items, starts, nitems, nchunks, grid, st, host_item);
       if (d == 1) launch_one<T, OP_DIFFUSE, 1>(items, starts, nitems, nchunks, grid, st, host_item);
@@ -2552,7 +2561,6 @@ unsigned op_count(int op, int d, const LevelView& L, const LevelView& F, const B
     case OP_SWEEP:
       n = (long long)sweep_units(b, d) * kBlock;  // one chunk per (column, chunk) unit
       break;
-    case OP_FRONTIER_DIFF: n = 24LL * L.acc_slots; break;
     case OP_BC: n = bc_elements(L, bc); break;
     case OP_COMMUP:  // one chunk per tile of the ghost hosts' shell
       n = cu_chunks(F.n, F.G) * kBlock;
