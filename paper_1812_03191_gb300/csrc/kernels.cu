@@ -1400,36 +1400,42 @@ __device__ __forceinline__ void el_bc(const LevelView& L, const int* bc, T V0, T
   if (!bc_element(L, bc, tid, c)) return;
   const int dst = (c[2] * L.s[1] + c[1]) * L.s[0] + c[0];
   const T V[3] = {V0, V1, V2};
+  // every field's source first, so that no load waits for a store
+  int how[5], flip[5];  // flip: the normal velocity changed sign
+  T fixed[5];
+  St<T> q[5];
 #pragma unroll
   for (int f = 0; f < 5; ++f) {
     int src[3] = {c[0], c[1], c[2]};
-    int how = 0, flip = 0;  // flip: the normal velocity changed sign
-    T fixed = T(0);
+    how[f] = flip[f] = 0;
+    fixed[f] = T(0);
 #pragma unroll
     for (int d = 2; d >= 0; --d) {
-      if (how == 3) continue;
+      if (how[f] == 3) continue;
       const int h = bc_source<T>(L.G, L.n[d], bc[2 * d], bc[2 * d + 1], f == F_VX + d, V[d],
-                                 src[d], fixed);
-      if (h == 2) flip = 1;
-      if (h) how = h;
+                                 src[d], fixed[f]);
+      if (h == 2) flip[f] = 1;
+      if (h) how[f] = h;
     }
-    if (!how) continue;
-    St<T>* q = (St<T>*)L.q[f];
+    if (how[f] == 1 || how[f] == 2)
+      q[f] = ((const St<T>*)L.q[f])[(src[2] * L.s[1] + src[1]) * L.s[0] + src[0]];
+  }
+#pragma unroll
+  for (int f = 0; f < 5; ++f) {
+    if (!how[f]) continue;
+    St<T>* out = (St<T>*)L.q[f];
     const T Vf = f >= F_VX ? V[f - F_VX] : T(0);
     if (f >= F_VX && bc_wraps(L, bc, f - F_VX)) {
       if (c[f - F_VX] == 0) continue;
       if (c[f - F_VX] == L.G + L.n[f - F_VX])
-        put(q, dst - c[f - F_VX] * L.st[f - F_VX], T(-1) * val(q, dst) + T(-2) * Vf);
+        put(out, dst - c[f - F_VX] * L.st[f - F_VX], T(-1) * val(out, dst) + T(-2) * Vf);
     }
-    const int cs = (src[2] * L.s[1] + src[1]) * L.s[0] + src[0];
-    if (how == 3) {
-      // (a flip found on a later axis than the fixed value's)
-      put(q, dst, flip ? -fixed - T(2) * Vf : fixed);
-    } else if (flip) {
-      put(q, dst, T(-1) * val(q, cs) + T(-2) * Vf);
-    } else {
-      q[dst] = q[cs];  // a copy keeps the stored value as it is
-    }
+    if (how[f] == 3)  // (a flip found on a later axis than the fixed value's)
+      put(out, dst, flip[f] ? -fixed[f] - T(2) * Vf : fixed[f]);
+    else if (flip[f])
+      put(out, dst, T(-1) * val(&q[f], 0) + T(-2) * Vf);
+    else
+      out[dst] = q[f];  // a copy keeps the stored value as it is
   }
 }
 
