@@ -109,12 +109,14 @@ __host__ __device__ constexpr int sweep_blocks(int esz, int d) {
 }
 __host__ __device__ inline int sweep_row_axis(int d) { return d == 1 ? 2 : 1; }
 __host__ __device__ inline int sweep_march_axis(int d) { return d == 0 ? 2 : d; }
-// double-float: planes of the march in flight, and the arrays of a plane
-constexpr int kSweepStages = 3;
+// the arrays of a plane; double-float: planes fetched ahead, and planes in the buffer (the
+// newest, two before it and those ahead)
 constexpr int kSweepArrays = 8;
-// values of the buffer of the planes in flight (FP32 keeps its one plane in registers)
-__host__ __device__ constexpr int sweep_ahead(int esz) {
-  return esz == 8 ? kSweepStages * kSweepArrays * kSweepThreads : kSweepThreads;
+constexpr int kSweepAhead = 2;
+constexpr int kSweepSlots = kSweepAhead + 3;
+// values of a block's buffer (FP32 keeps its planes in registers)
+__host__ __device__ constexpr int sweep_buffer(int esz) {
+  return esz == 8 ? kSweepSlots * kSweepArrays * kSweepThreads : kSweepThreads;
 }
 // positions a warp owns, and halo positions of a row
 __host__ __device__ constexpr int sweep_own(int d) { return d == 0 ? 27 : 31; }

@@ -884,48 +884,67 @@ __device__ __forceinline__ void stb(P* base, unsigned o, C v) {
   st((P*)((char*)base + o), 0, v);
 }
 
-// The planes to come, fetched ahead.  FP32: one plane, in registers (copies into shared
-// memory measured the same).  Double-float: kSweepStages planes by asynchronous copies
-// into shared memory, each thread's values in its own column of the buffer (so no
-// barrier): registers for them would cost a block per SM (y, z: 132 -> 118 us at 136^3,
-// with the unnormalised sums).
+// The planes of a march as loaded: the newest, the two before it, and those to come.
+//   FP32: in registers, one plane ahead (shared memory measured the same to 1 % slower,
+// with four or five blocks an SM alike).
 template <class C>
-struct Ahead {
-  static constexpr int NS = 2;
-  C v[kSweepArrays];
-  __device__ __forceinline__ explicit Ahead(C*) {}
+struct Planes {
+  static constexpr int kAhead = 1;
+  C q[3][kSweepArrays], to_come[kSweepArrays];
+  __device__ __forceinline__ explicit Planes(C*) {}
   template <class P>
   __device__ __forceinline__ void fetch(int a, const P* base, unsigned o) {
-    v[a] = ldb(base, o);
+    to_come[a] = ldb(base, o);
   }
+  __device__ __forceinline__ void clear(int a) { to_come[a] = C(0.f); }
   __device__ __forceinline__ void commit() {}
-  __device__ __forceinline__ void take(C (&q)[kSweepArrays]) {
+  __device__ __forceinline__ void advance() {
 #pragma unroll
-    for (int a = 0; a < kSweepArrays; ++a) q[a] = v[a];
+    for (int a = 0; a < kSweepArrays; ++a) {
+      q[2][a] = q[1][a];
+      q[1][a] = q[0][a];
+      q[0][a] = to_come[a];
+    }
   }
+  // array a of the plane `back` before the newest
+  __device__ __forceinline__ C get(int back, int a) const { return q[back][a]; }
 };
+//   Double-float: in shared memory, kSweepAhead planes ahead by asynchronous copies, each
+// thread's values in its own column of the buffer (so no barrier).  In registers they
+// would take 46: with the planes to come alone in shared memory the march needed 168 and
+// spilled, 138 us a sweep of 5 x 128^3 against 124 now with 152 (four blocks of 128
+// registers spill again, 126).
 template <>
-struct Ahead<df64> {
-  static constexpr int NT = kSweepThreads, NS = kSweepStages;
-  df64* buf;  // [stage][array][thread], at this thread
-  int in = 0, out = 0;
-  __device__ __forceinline__ explicit Ahead(df64* b) : buf(b) {}
+struct Planes<df64> {
+  static constexpr int kAhead = kSweepAhead, NT = kSweepThreads, SLOT = kSweepArrays * NT;
+  df64* buf;  // [slot][array][thread], at this thread
+  // slots to fetch to, of the newest plane and of the two before (before the first plane
+  // they name slots whose values nothing that is kept depends on)
+  int in = 0, s0 = (kSweepSlots - 1) * SLOT, s1 = 0, s2 = 0;
+  __device__ __forceinline__ explicit Planes(df64* b) : buf(b) {}
+  static __device__ __forceinline__ int next(int s) {
+    return s == (kSweepSlots - 1) * SLOT ? 0 : s + SLOT;
+  }
   template <class P>
   __device__ __forceinline__ void fetch(int a, const P* base, unsigned o) {
-    const unsigned s = (unsigned)__cvta_generic_to_shared(buf + (in * kSweepArrays + a) * NT);
+    const unsigned s = (unsigned)__cvta_generic_to_shared(buf + in + a * NT);
     asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(s), "l"((const char*)base + o)
                  : "memory");
   }
+  __device__ __forceinline__ void clear(int a) { buf[in + a * NT] = df64(0.f); }
   __device__ __forceinline__ void commit() {
     asm volatile("cp.async.commit_group;" ::: "memory");
-    in = in + 1 == NS ? 0 : in + 1;
+    in = next(in);
   }
-  // the oldest plane in flight, once it has arrived
-  __device__ __forceinline__ void take(df64 (&q)[kSweepArrays]) {
-    asm volatile("cp.async.wait_group %0;" ::"n"(NS - 1) : "memory");
-#pragma unroll
-    for (int a = 0; a < kSweepArrays; ++a) q[a] = buf[(out * kSweepArrays + a) * NT];
-    out = out + 1 == NS ? 0 : out + 1;
+  // the oldest plane in flight has arrived and becomes the newest
+  __device__ __forceinline__ void advance() {
+    asm volatile("cp.async.wait_group %0;" ::"n"(kAhead - 1) : "memory");
+    s2 = s1;
+    s1 = s0;
+    s0 = next(s0);
+  }
+  __device__ __forceinline__ df64 get(int back, int a) const {
+    return buf[(back == 0 ? s0 : back == 1 ? s1 : s2) + a * NT];
   }
 };
 
@@ -958,44 +977,42 @@ __device__ __forceinline__ void sweep_march(const Item<T>& it, int x, int row, b
   const int f0 = L.G, f1 = L.G + L.n[d];
 
   // fetch plane p: this row's values and, of the row below, rho and v_d
-  Ahead<C> ah(buf);
+  Planes<C> pl(buf);
   const int r_end = m1 + 2;
   auto fetch = [&](int p) {
     if (p < r_end && (!EDGE || (unsigned)p < (unsigned)sM)) {
       const unsigned c = c0 + (unsigned)p * stM, b = cb + (unsigned)p * stM;
-      ah.fetch(0, rhoS, c);
-      ah.fetch(1, eS, c);
-      ah.fetch(2, vd, c);
+      pl.fetch(0, rhoS, c);
+      pl.fetch(1, eS, c);
+      pl.fetch(2, vd, c);
 #pragma unroll
-      for (int m = 0; m < 3; ++m) ah.fetch(3 + m, piS(m), c);
-      ah.fetch(6, rhoS, b);
-      ah.fetch(7, vd, b);
+      for (int m = 0; m < 3; ++m) pl.fetch(3 + m, piS(m), c);
+      pl.fetch(6, rhoS, b);
+      pl.fetch(7, vd, b);
+    } else if (EDGE && p < r_end) {
+#pragma unroll
+      for (int a = 0; a < kSweepArrays; ++a) pl.clear(a);
     }
-    ah.commit();
+    pl.commit();
   };
 
   // windows at step r (plane r is the newest): x1, x2 the values of planes r-1, r-2, dx0
   // the difference of planes r and r-1, dx1, dx2 the two before
   const C z = C(0.f);
-  C r1 = z, r2 = z, dr1 = z, dr2 = z;                       // rho
+  C dr1 = z, dr2 = z, db1 = z, db2 = z;                     // rho; of the row below
   C e1 = z, e2 = z, de1 = z, de2 = z;                       // e/rho
-  C b1 = z, db1 = z, db2 = z, b2 = z;                       // rho, row below
   C w1[3] = {z, z, z}, w2[3] = {z, z, z};                   // Pi/rho_face - V
   C dw1[3] = {z, z, z}, dw2[3] = {z, z, z};
-  C en1 = z, en2 = z, v1 = z, v2 = z, vb1 = z;              // e, v_d, v_d of the row below
-  C p1[3] = {z, z, z}, p2[3] = {z, z, z};                   // momenta
   C F2 = z, E2 = z, Pp[3] = {z, z, z};                      // fluxes of the face before
-  for (int k = 0; k < Ahead<C>::NS - 1; ++k) fetch(m0 - 3 + k);
+  for (int k = 0; k < Planes<C>::kAhead; ++k) fetch(m0 - 3 + k);
 #pragma unroll 1
   for (int r = m0 - 3; r < r_end; ++r) {
-    C q[kSweepArrays];
-    if (sizeof(T) == 8) fetch(r + Ahead<C>::NS - 1);
-    ah.take(q);
-    if (sizeof(T) == 4) fetch(r + 1);
-    C rc = q[0], ec = q[1], vc = q[2], rb = q[6], vb = q[7];
-    C pc[3] = {q[3], q[4], q[5]};
-    if (EDGE && (unsigned)r >= (unsigned)sM)
-      rc = ec = vc = rb = vb = pc[0] = pc[1] = pc[2] = z;
+    // a slot is free again once the plane three before is done with
+    pl.advance();
+    fetch(r + Planes<C>::kAhead);
+    const C rc = pl.get(0, 0), ec = pl.get(0, 1), rb = pl.get(0, 6);
+    const C r1 = pl.get(1, 0), b1 = pl.get(1, 6);
+    const C pc[3] = {pl.get(0, 3), pl.get(0, 4), pl.get(0, 5)};
     // e/rho and Pi/rho_face - V = (dPi - V drf)/(rho0 + drf) of plane r
     const C ep = eps_dev(ec, rc, bg);
     const C rx = shfl_up(rc, 1);
@@ -1015,6 +1032,7 @@ __device__ __forceinline__ void sweep_march(const Item<T>& it, int x, int row, b
       // mass and energy flux of face r - 1, and the mass flux of the row below
       const int f = r - 1;
       const bool ok = !EDGE || (f >= 2 && f < sM - 1);
+      const C r2 = pl.get(2, 0), b2 = pl.get(2, 6), v1 = pl.get(1, 2), vb1 = pl.get(1, 7);
       C Fb = z;
       if (ok) {
         const C u = add_k(v1, bg.V[d]), ub = add_k(vb1, bg.V[d]);
@@ -1049,7 +1067,7 @@ __device__ __forceinline__ void sweep_march(const Item<T>& it, int x, int row, b
           P[RA] = ky_add(bg.V[RA], Fe, mul_u(ws, add_k(Fe, F0)));
         }
         if (!EDGE || (r - 2 >= 2 && r - 2 < sM - 2)) {
-          const C uc = add_k(halve(v2 + v1), bg.V[d]);
+          const C uc = add_k(halve(pl.get(2, 2) + v1), bg.V[d]);
           const C Fc = halve(add_u(F2, F1));
           const C ws = upwind_d(w2[d], w1[d], dw2[d], dw1[d], dw0[d], uc, mul_u(uc, dtdx));
           P[d] = ky_add(bg.V[d], Fc, mul_u(ws, add_k(Fc, F0)));
@@ -1060,7 +1078,7 @@ __device__ __forceinline__ void sweep_march(const Item<T>& it, int x, int row, b
       if (u2 >= m0 && own) {
         const unsigned c = c0 + (unsigned)u2 * stM;
         const bool upd = !EDGE || (u2 >= 2 && u2 < sM - 2);
-        C rv = r2, ev = en2;
+        C rv = r2, ev = pl.get(2, 1);
         if (upd) {
           C Flo = F2, Fhi = F1, Elo = E2, Ehi = E1;
           if (L.has_child && near_frontier(L, d, u2)) {
@@ -1077,7 +1095,7 @@ __device__ __forceinline__ void sweep_march(const Item<T>& it, int x, int row, b
         stb(eD, c, ev);
 #pragma unroll
         for (int m = 0; m < 3; ++m) {
-          C pv = p2[m];
+          C pv = pl.get(2, 3 + m);
           // P_d of cells r-3, r-2; the others' of planes r-2, r-1
           if (!EDGE || (upd && (m == d ? u2 >= 3 : m == 0 ? x >= 1 : row >= 1)))
             pv = pv - mul_u(sub_u(P[m], Pp[m]), iv);
@@ -1088,14 +1106,11 @@ __device__ __forceinline__ void sweep_march(const Item<T>& it, int x, int row, b
       for (int m = 0; m < 3; ++m) Pp[m] = P[m];
     }
     F2 = F1; E2 = E1;
-    r2 = r1; r1 = rc; dr2 = dr1; dr1 = dr0;
+    dr2 = dr1; dr1 = dr0; db2 = db1; db1 = db0;
     e2 = e1; e1 = ep; de2 = de1; de1 = de0;
-    b2 = b1; b1 = rb; db2 = db1; db1 = db0;
-    en2 = en1; en1 = ec; v2 = v1; v1 = vc; vb1 = vb;
 #pragma unroll
     for (int m = 0; m < 3; ++m) {
       w2[m] = w1[m]; w1[m] = w0[m]; dw2[m] = dw1[m]; dw1[m] = dw0[m];
-      p2[m] = p1[m]; p1[m] = pc[m];
     }
   }
 }
@@ -1126,30 +1141,30 @@ __device__ __forceinline__ void sweep_x(const Item<T>& it, int x, int row, bool 
   const bool okF = !EDGE || (x >= 2 && x < sx - 1);
   const C z = C(0.f);
 
-  Ahead<C> ah(buf);
+  Planes<C> pl(buf);
   auto fetch = [&](int p) {
     if (p < m1 && (!EDGE || p >= 0)) {
       const unsigned c = c0 + (unsigned)p * stM, b = cb + (unsigned)p * stM;
-      ah.fetch(0, rhoS, c);
-      ah.fetch(1, eS, c);
+      pl.fetch(0, rhoS, c);
+      pl.fetch(1, eS, c);
 #pragma unroll
-      for (int m = 0; m < 3; ++m) ah.fetch(2 + m, (const St<T>*)L.q[F_VX + m], c);
-      ah.fetch(5, rhoS, b);
-      ah.fetch(6, (const St<T>*)L.q[F_VX], b);
+      for (int m = 0; m < 3; ++m) pl.fetch(2 + m, (const St<T>*)L.q[F_VX + m], c);
+      pl.fetch(5, rhoS, b);
+      pl.fetch(6, (const St<T>*)L.q[F_VX], b);
+    } else if (EDGE && p < m1) {
+#pragma unroll
+      for (int a = 0; a < kSweepArrays; ++a) pl.clear(a);
     }
-    ah.commit();
+    pl.commit();
   };
-  for (int k = 0; k < Ahead<C>::NS - 1; ++k) fetch(m0 - 1 + k);
+  for (int k = 0; k < Planes<C>::kAhead; ++k) fetch(m0 - 1 + k);
   C rp = z, vp = z, Fp = z;  // rho, v_x, F of the plane before
 #pragma unroll 1
   for (int p = m0 - 1; p < m1; ++p) {
-    C q[kSweepArrays];
-    if (sizeof(T) == 8) fetch(p + Ahead<C>::NS - 1);
-    ah.take(q);
-    if (sizeof(T) == 4) fetch(p + 1);
-    C rc = q[0], ec = q[1], rb = q[5], vb = q[6];
-    C w[3] = {q[2], q[3], q[4]};
-    if (EDGE && p < 0) rc = ec = rb = vb = w[0] = w[1] = w[2] = z;
+    pl.advance();
+    fetch(p + Planes<C>::kAhead);
+    const C rc = pl.get(0, 0), ec = pl.get(0, 1), rb = pl.get(0, 5), vb = pl.get(0, 6);
+    const C w[3] = {pl.get(0, 2), pl.get(0, 3), pl.get(0, 4)};
     const C vc = w[0];
     const C r_m1 = shfl_up(rc, 1);
     C Fv = z, Ev = z, Fb = z;
@@ -2409,10 +2424,10 @@ __global__ void __launch_bounds__(kBlock, 3) k_reduce(const Item<T>* __restrict_
 template <class T, int D>
 __global__ void __launch_bounds__(kSweepThreads, sweep_blocks((int)sizeof(T), D))
     k_sweep_single(const Item<T> it) {
-  __shared__ Arith<T> s_ahead[sweep_ahead((int)sizeof(T))];
+  __shared__ Arith<T> s_planes[sweep_buffer((int)sizeof(T))];
   pdl_enter();
   if (skipped(it)) return;
-  el_sweep<T, D>(it, blockIdx.x, s_ahead + threadIdx.x);
+  el_sweep<T, D>(it, blockIdx.x, s_planes + threadIdx.x);
   pdl_exit();
 }
 
@@ -2420,7 +2435,7 @@ template <class T, int D>
 __global__ void __launch_bounds__(kSweepThreads, sweep_blocks((int)sizeof(T), D))
     k_sweep_batch(const Item<T>* __restrict__ items, const unsigned* __restrict__ starts,
                   int nitems, unsigned nchunks) {
-  __shared__ Arith<T> s_ahead[sweep_ahead((int)sizeof(T))];
+  __shared__ Arith<T> s_planes[sweep_buffer((int)sizeof(T))];
   __shared__ __align__(16) unsigned char s_raw[sizeof(Item<T>)];
   const Item<T>& it = *reinterpret_cast<const Item<T>*>(s_raw);
   pdl_enter();
@@ -2445,7 +2460,7 @@ __global__ void __launch_bounds__(kSweepThreads, sweep_blocks((int)sizeof(T), D)
       __syncthreads();
       cur = lo;
     }
-    if (!skipped(it)) el_sweep<T, D>(it, ch - starts[cur], s_ahead + threadIdx.x);
+    if (!skipped(it)) el_sweep<T, D>(it, ch - starts[cur], s_planes + threadIdx.x);
     __syncthreads();
   }
   pdl_exit();
