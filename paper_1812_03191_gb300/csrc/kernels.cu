@@ -66,8 +66,10 @@ __device__ __forceinline__ int cidx(const LevelView& L, int i, int j, int k) {
 // q <- q + r(a - b q) (Markstein, IBM J. Res. Dev. 34 (1990)): the corrected
 // quotient's error is the square of the refined reciprocal's plus the final
 // rounding, within one ulp for the normal, non-zero divisors used here (densities,
-// 1 + a, and the sum of two same-signed slopes).  FP32: the fast reciprocal-based
-// divide.
+// 1 + a, and the sum of two same-signed slopes).  FP32: the product with the hardware
+// reciprocal estimate (within one ulp; __fdividef is the same for these divisors, but
+// guards against ones beyond 2^126 with some four instructions more, ten times a cell in a
+// sweep).
 __device__ __forceinline__ double hdiv(double a, double b) {
   double r;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(b));
@@ -75,12 +77,12 @@ __device__ __forceinline__ double hdiv(double a, double b) {
   double q = a * r;
   return fma(r, fma(-b, q, a), q);
 }
-__device__ __forceinline__ float hdiv(float a, float b) { return __fdividef(a, b); }
+__device__ __forceinline__ float hdiv(float a, float b) { return a * rcp_est(b); }
 __device__ __forceinline__ df64 hdiv(df64 a, df64 b) { return a / b; }
 // product and quotient whose result only feeds more arithmetic: in double-float left
 // without the final renormalisation (mul_u, div_u in df64.h), in FP32 the plain ones
 __device__ __forceinline__ float mul_u(float a, float b) { return a * b; }
-__device__ __forceinline__ float div_u(float a, float b) { return __fdividef(a, b); }
+__device__ __forceinline__ float div_u(float a, float b) { return a * rcp_est(b); }
 // likewise the sum, the difference and p - a of a float p (add_u, sub_u, fsub_u there)
 __device__ __forceinline__ float add_u(float a, float b) { return a + b; }
 __device__ __forceinline__ float sub_u(float a, float b) { return a - b; }
@@ -865,12 +867,13 @@ __device__ __forceinline__ df64 shfl_dn(df64 v, int k) {
 }
 
 // the upwind value (upwind_v) from the two sides' values and the differences
-// dm = q(-1) - q(-2), dc = q(0) - q(-1), dp = q(1) - q(0)
+// dm = q(-1) - q(-2), dc = q(0) - q(-1), dp = q(1) - q(0).  The limiter takes dc and one
+// of the others, and is symmetric in the two: one selection.
 template <class C>
 __device__ __forceinline__ C upwind_d(C qm, C q0, C dm, C dc, C dp, C u, C cour) {
   const bool up = gt0(u);
-  return add_u(up ? qm : q0, mul_u(fsub_u(up ? 1.f : -1.f, cour),
-                                   hslope(up ? dm : dc, up ? dc : dp)));
+  return add_u(up ? qm : q0,
+               mul_u(fsub_u(up ? 1.f : -1.f, cour), hslope(dc, up ? dm : dp)));
 }
 
 // element access by byte offset from a base that is the same for the whole warp (offsets
