@@ -694,26 +694,18 @@ struct Builder {
     return it;
   }
 
-  // Planes per chunk of a fused sweep over box b.  A context: as many chunks as leave
-  // every block resident at once, but at least 4 planes (x sweep: 1) each, since a chunk
-  // repeats 5 (1) (levels of 32^3 to 64^3: 6 planes ran up to 8 % slower per coarse
-  // step, 1 to 3 planes no faster).  A pool: its launches hold every run's sweep, so the
-  // chunk is what gives about 2000 blocks in all, within 8 and 32 planes (24 runs of 32^3
-  // to 96^3: 8.06 ms a step with 6 planes, 7.26 with 24, 7.40 with 40; 16 runs of 24^3 to
-  // 32^3: 0.99 with 12, 1.17 with 24).
+  // Box::zc of a fused sweep over box b.  A context's sweep has the device to itself
+  // (sweep_split).  A pool's launches hold every run's sweep, so the chunk is what gives
+  // about 2000 blocks in all, within 8 and 32 planes (24 runs of 32^3 to 96^3: 8.06 ms a
+  // step with 6 planes, 7.26 with 24, 7.40 with 40; 16 runs of 24^3 to 32^3: 0.99 with 12,
+  // 1.17 with 24).
   int sweep_chunk(const Box& b, int d) const {
-    const int mu = sweep_march_axis(d), nm = b.hi[mu] - b.lo[mu];
-    int zc;
-    if (pool) {
-      const long long fit = pool_cells / (sweep_own(1) * (kSweepThreads / 32)) / 2000;
-      zc = (int)std::min<long long>(std::max<long long>(fit, 8), 32);
-      if (d == 0) zc /= 2;
-    } else {
-      const int slots = sm_count * sweep_blocks((int)sizeof(T), d);
-      const int chunks = std::max(1, slots / std::max(1, sweep_columns(b, d)));
-      zc = std::max((nm + chunks - 1) / chunks, d == 0 ? 1 : 4);
-    }
-    return std::min(nm, zc);
+    if (!pool)
+      return sweep_split(b, d, sweep_blocks((int)sizeof(T), d), sm_count, sizeof(T) == 8);
+    const int mu = sweep_march_axis(d);
+    const long long fit = pool_cells / (sweep_own(1) * (kSweepThreads / 32)) / 2000;
+    const int zc = (int)std::min<long long>(std::max<long long>(fit, 8), 32);
+    return std::min(b.hi[mu] - b.lo[mu], d == 0 ? zc / 2 : zc);
   }
 
   // margin boxes (active cells +- margin) unless verifying with whole arrays or the

@@ -1,8 +1,9 @@
 // kernels.cu -- sm_103a kernels of one level step of the nested-mesh solver
 // (Velasco Romero & Masset 2018, Sec. 3) and of the inter-level operators.
 //
-// Each stencil kernel is one thread per element of a box (flattened, x fastest, so
-// consecutive threads touch consecutive addresses).  A kernel applies its operator
+// Each stencil kernel but the fused transport sweeps (whose lanes march through a box) is
+// one thread per element of a box (flattened, x fastest, so consecutive threads touch
+// consecutive addresses).  A kernel applies its operator
 // to the elements of the box where its stencil fits inside the padded array; the
 // host picks the box (the active cells plus the margin whose values can still reach
 // them before the next ghost fill).  T is the state type (double, or float for the
@@ -851,10 +852,13 @@ __device__ __forceinline__ void frontier_fluxes(const LevelView& L, int d, const
 // no element that is needed later depends on them.
 //   EDGE: the box reaches the ends of the array, where the stencils do not fit (faces 0,
 // 1 and the last along d, face 0 of the other axes).
-//   Bound by instruction issue.  Measured at a 136^3 box (ncu, GB300): FP32 state x 40.5,
-// y 36.9, z 36.8 us, 352 / 314 / 313 lane instructions per cell, against 54-63 us for the
-// earlier form (blocks of 9 warps, one barrier a plane, 363-400 instructions);
-// double-float 137 / 119 / 117 us, 1330 / 1163 / 1162 instructions.
+//   Bound by instruction issue (FP32 65-74 % of the issue slots, double-float 73-75 %).
+// Measured at a box of 136^3 (ncu, GB300): FP32 state x 33.0, y 32.1, z 32.4 us and 261 /
+// 276 / 266 thread instructions per cell, where an earlier form with blocks of 9 warps and
+// a barrier a plane took 363-400; double-float x 136, y 94, z 97 us and 1097 / 939 / 935
+// instructions.  Over a coarse step of 5 x 128^3 a sweep takes 40 us in FP32 and 122 in
+// double-float, where that form took 68 us in FP32 and the four separate kernels 171 in
+// double-float.
 __device__ __forceinline__ float shfl_up(float v, int k) {
   return __shfl_up_sync(0xffffffffu, v, k);
 }
@@ -1294,18 +1298,16 @@ __device__ __forceinline__ void sweep_x(const Item<T>& it, int x, int row, bool 
   }
 }
 
+// planes [m0, m1) of a column
 template <class T, int d>
-__device__ __forceinline__ void el_sweep(const Item<T>& it, unsigned unit,
-                                         Arith<T>* __restrict__ buf) {
-  constexpr int RA = d == 1 ? 2 : 1, MU = d == 0 ? 2 : d;
+__device__ __forceinline__ void sweep_column(const Item<T>& it, int col, int m0, int m1,
+                                             Arith<T>* __restrict__ buf) {
+  constexpr int RA = d == 1 ? 2 : 1;
   const Box& b = it.b;
-  const int ncol = sweep_columns(b, d);
-  const int chunk = (int)unit / ncol, col = (int)unit - chunk * ncol;
   SweepLane p;
   if (!sweep_lane(b, d, col * (kSweepThreads / 32) + (int)(threadIdx.x >> 5),
                   (int)(threadIdx.x & 31), p))
     return;
-  const int m0 = b.lo[MU] + chunk * b.zc, m1 = min(m0 + b.zc, b.hi[MU]);
   if (d == 0) {
     if (b.lo[0] >= 3 && b.hi[0] <= it.L.s[0] - 2 && b.lo[1] >= 1 && m0 >= 1)
       sweep_x<T, false>(it, p.x, p.row, p.mine, m0, m1, buf);
@@ -1316,6 +1318,31 @@ __device__ __forceinline__ void el_sweep(const Item<T>& it, unsigned unit,
       sweep_march<T, d == 0 ? 1 : d, false>(it, p.x, p.row, p.mine && p.x >= b.lo[0], m0, m1, buf);
     else
       sweep_march<T, d == 0 ? 1 : d, true>(it, p.x, p.row, p.mine && p.x >= b.lo[0], m0, m1, buf);
+  }
+}
+
+// a unit of a sweep; ENDS: the columns are laid end to end (Box::zc < 0), a form of its own
+// because one form for both ran 0.6 % slower where chunks are taken (3 x 64^3 FP64 762 and
+// 766 us a coarse step)
+template <class T, int d, bool ENDS>
+__device__ __forceinline__ void el_sweep(const Item<T>& it, unsigned unit,
+                                         Arith<T>* __restrict__ buf) {
+  constexpr int MU = d == 0 ? 2 : d;
+  const Box& b = it.b;
+  if (ENDS) {
+    const int nm = b.hi[MU] - b.lo[MU];
+    int pos, end;
+    sweep_unit(b, d, (int)unit, pos, end);
+    while (pos < end) {
+      const int col = pos / nm, m0 = b.lo[MU] + pos - col * nm;
+      const int m1 = min(m0 + end - pos, b.hi[MU]);
+      sweep_column<T, d>(it, col, m0, m1, buf);
+      pos += m1 - m0;
+    }
+  } else {
+    const int ncol = sweep_columns(b, d), chunk = (int)unit / ncol;
+    const int m0 = b.lo[MU] + chunk * b.zc;
+    sweep_column<T, d>(it, (int)unit - chunk * ncol, m0, min(m0 + b.zc, b.hi[MU]), buf);
   }
 }
 
@@ -2462,13 +2489,13 @@ __global__ void __launch_bounds__(kBlock, 3) k_reduce(const Item<T>* __restrict_
 
 // Fused sweep: one block per (column, chunk) unit; the work-list form stages the item as
 // k_batch does.
-template <class T, int D>
+template <class T, int D, bool ENDS>
 __global__ void __launch_bounds__(kSweepThreads, sweep_blocks((int)sizeof(T), D))
     k_sweep_single(const Item<T> it) {
   __shared__ Arith<T> s_planes[sweep_buffer((int)sizeof(T))];
   pdl_enter();
   if (skipped(it)) return;
-  el_sweep<T, D>(it, blockIdx.x, s_planes + threadIdx.x);
+  el_sweep<T, D, ENDS>(it, blockIdx.x, s_planes + threadIdx.x);
   pdl_exit();
 }
 
@@ -2501,7 +2528,7 @@ __global__ void __launch_bounds__(kSweepThreads, sweep_blocks((int)sizeof(T), D)
       __syncthreads();
       cur = lo;
     }
-    if (!skipped(it)) el_sweep<T, D>(it, ch - starts[cur], s_planes + threadIdx.x);
+    if (!skipped(it)) el_sweep<T, D, false>(it, ch - starts[cur], s_planes + threadIdx.x);
     __syncthreads();
   }
   pdl_exit();
@@ -2529,9 +2556,14 @@ template <class T, int D>
 static void launch_sweep(const Item<T>* items, const unsigned* starts, int nitems,
                          unsigned nchunks, unsigned grid, cudaStream_t st,
                          const Item<T>* host_item) {
+  if constexpr (sizeof(T) == 8)
+    if (nitems == 1 && host_item && host_item->b.zc < 0) {
+      launch_pdl(k_sweep_single<T, D, true>, nchunks, kSweepThreads, st, *host_item);
+      return;
+    }
   if (nitems == 1 && host_item)
-    launch_pdl(k_sweep_single<T, D>, nchunks, kSweepThreads, st, *host_item);
-  else
+    launch_pdl(k_sweep_single<T, D, false>, nchunks, kSweepThreads, st, *host_item);
+  else  // pools, whose items have chunks (Box::zc > 0)
     launch_pdl(k_sweep_batch<T, D>, grid, kSweepThreads, st, items, starts, nitems, nchunks);
 }
 
