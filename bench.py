@@ -128,7 +128,10 @@ class ClockSampler:
 
 # --------------------------------------------------------------- algorithmic bytes
 # Arrays each stencil kernel reads + writes once per element of its box (the
-# compulsory traffic of the kernel as designed, neighbour reuse assumed cached).
+# compulsory traffic of the kernel as designed, neighbour reuse assumed cached).  The
+# boxes counted (level_step_boxes) are the active cells and the whole margin of the level
+# step; the library gives each operator only the margin that the next ones read, so these
+# bytes are an upper bound, 1.14 times the swept elements' for levels of 128^3.
 ARRAYS_PER_ELEM = {
     "source": 12,        # rho, e, phi, v3 -> v3, pi3
     "compress_lum": 8,   # e, v3, rho, lumw -> e, e/rho
@@ -139,8 +142,8 @@ ARRAYS_PER_ELEM = {
     "tflux": 5,          # rho, e/rho, v_d -> F, E
     "tmom": 8,           # w3, F, v_d -> P3
     "tupdate": 15,       # F, E, P3, rho, e, pi3 -> rho, e, pi3
-    "vrec_source": 9,    # rho, e, phi, pi3 -> v3 (after fused sweeps also -> rho, e)
-    "sweep": 11,         # fused sweep: rho, e, pi3, v_d -> rho, e, pi3
+    "vrec_source": 9,    # rho, e, phi, pi3 -> v3 (counted + 2 after fused sweeps)
+    "sweep": 11,         # fused sweep, the default: rho, e, pi3, v_d -> rho, e, pi3
 }
 
 
@@ -799,8 +802,7 @@ def main():
     ap.add_argument("--no-cpu", action="store_true")
     ap.add_argument("--transport", default="auto", choices=["auto", "separate", "fused"],
                     help="transport kernels: fused sweeps or separate kernels (default: "
-                         "the library's choice: fused sweeps for the FP32 state in pools and "
-                         "on levels of at least 512 Ki cells)")
+                         "the library's choice, fused sweeps)")
     ap.add_argument("--tiles", default="auto", choices=["auto", "flat"],
                     help="tile shapes of the stencil launches: autotuned (before the "
                          "warm-up, untimed) or flat enumeration")
@@ -849,7 +851,6 @@ def main():
     flush = torch.empty(256 * 1024 * 1024 // 4, dtype=torch.float32, device="cuda")
     transport = {"auto": binding.TRANSPORT_AUTO, "separate": binding.TRANSPORT_SEPARATE,
                  "fused": binding.TRANSPORT_FUSED}[args.transport]
-    n3 = cfg["n"] ** 3 if isinstance(cfg["n"], int) else int(np.prod(cfg["n"]))
     peak, peak_kind = peaks()
 
     # measured FP64 peak (the FP64 kernels are bound by the FP64 pipe), clocks sampled
@@ -862,8 +863,7 @@ def main():
                           cfg["params"], precision=pr, device=local, stream=stream.cuda_stream)
         sim.set_transport(transport)
         fused = transport == binding.TRANSPORT_FUSED or (
-            transport == binding.TRANSPORT_AUTO and pr == binding.DF_FP32_STATE
-            and n3 >= 512 * 1024)  # the library's per-level choice
+            transport == binding.TRANSPORT_AUTO)  # the library's choice
         return sim, fused
 
     sim, fused = make(prec)
