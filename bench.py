@@ -142,20 +142,21 @@ ARRAYS_PER_ELEM = {
     "tflux": 5,          # rho, e/rho, v_d -> F, E
     "tmom": 8,           # w3, F, v_d -> P3
     "tupdate": 15,       # F, E, P3, rho, e, pi3 -> rho, e, pi3
-    "vrec_source": 9,    # rho, e, phi, pi3 -> v3 (counted + 2 after fused sweeps)
+    "vrec_source": 9,    # rho, e, phi, pi3 -> v3
     "sweep": 11,         # fused sweep, the default: rho, e, pi3, v_d -> rho, e, pi3
 }
 
 
-
-# DRAM bytes (read + write) per box element of a launch, from the ncu captures in
-# profiles/ (k_sweep_fused_precision_5x128_fp32.md: fused sweeps, 144^3 box,
-# 80.2 / 99.5 / 85.0 MB; k_tmom_df64_nested_3x64.md: double-float momentum fluxes, 80^3
-# box, 20.09 / 20.09 / 13.47 MB, a smaller case of the same kernel, whose traffic
-# grows with the box); `traffic` scales them to the mean box of the timed launches.
-# A kernel without a capture of its current code reports null.
+# DRAM bytes (read + write) of a launch per element of its level step's box, from the ncu
+# captures in profiles/ (k_sweep_fused_precision_5x128_fp32.md: fused sweeps of a 144^3 box,
+# 74.3 / 89.4 / 85.4 MB in FP32 and 223.7 / 224.3 / 202.4 MB in FP64; k_tmom_df64_nested_3x64.md:
+# double-float momentum fluxes of the separate transport kernels, 80^3 box, 20.09 / 20.09 /
+# 13.47 MB, a smaller case of the same kernel, whose traffic grows with the box); `traffic`
+# scales them to the mean box of the timed launches.  A kernel without a capture of its
+# current code reports null.
 _TMOM_DF64 = (20.0865e6 + 20.0840e6 + 13.4705e6) / 3 / 80**3
-TRAFFIC_PER_ELEM = {("precision_5x128^3", 4, "sweep"): (80.2e6 + 99.5e6 + 85.0e6) / 3 / 144**3,
+TRAFFIC_PER_ELEM = {("precision_5x128^3", 4, "sweep"): (74.3e6 + 89.4e6 + 85.4e6) / 3 / 144**3,
+                    ("precision_5x128^3", 8, "sweep"): (223.7e6 + 224.3e6 + 202.4e6) / 3 / 144**3,
                     ("precision_5x128^3", 8, "tmom"): _TMOM_DF64,
                     ("nested_3x64^3_fp64", 8, "tmom"): _TMOM_DF64}
 
@@ -175,8 +176,7 @@ def bytes_per_launch(cfg, kind, esz, fused=False):
     boxes = level_step_boxes(cfg)
     n, G = cfg["n"], cfg["G"]
     if kind in ARRAYS_PER_ELEM:
-        arrays = ARRAYS_PER_ELEM[kind] + (2 if fused and kind == "vrec_source" else 0)
-        arrays += 1 if kind == "diffuse" and not fused else 0
+        arrays = ARRAYS_PER_ELEM[kind] + (1 if kind == "diffuse" and not fused else 0)
         return arrays * esz * sum(boxes) / len(boxes)
     if kind == "commup":  # write every fine ghost element, read each coarse host once
         return 5 * esz * (((n + 2 * G) ** 3 - n**3) + (n // 2 + G + 2) ** 3)
@@ -365,8 +365,7 @@ def run_batched(args):
             continue
         boxes = level_step_boxes(dict(n=r["n"], G=r["G"], n_levels=r["n_levels"]))
         mult = 3 if dom in ("tprep", "tflux", "tmom", "tupdate", "sweep") else 1
-        arrays = ARRAYS_PER_ELEM[dom] + (2 if dom == "vrec_source" and swept else 0)
-        per_step_bytes += arrays * esz * sum(boxes) * mult
+        per_step_bytes += ARRAYS_PER_ELEM[dom] * esz * sum(boxes) * mult
     dom_ms, dom_n = kinds[dom]
     achieved = per_step_bytes * args.steps / (dom_ms / 1e3) / 1e9
     peak, peak_kind = peaks()
@@ -568,12 +567,8 @@ def run_serving(args):
     srv.close()
     seq64, summ64 = S.serve_sequential(reqs, budget, precision=binding.DF_FP64, tol=1e-3,
                                        step_cap=args.step_cap, keep_history=True)
-    # one run alone is faster with the separate transport kernels than with the fused
-    # sweeps (too few blocks per sweep on these small levels); the FP32 baseline uses
-    # them, so that the batching gain is not overstated
     seq32, summ32 = S.serve_sequential(reqs, budget, precision=binding.DF_FP32_STATE, tol=1e-3,
-                                       step_cap=args.step_cap,
-                                       transport=binding.TRANSPORT_SEPARATE)
+                                       step_cap=args.step_cap)
     # FP32-state error of each served result against the FP64 run of the same request
     # at the same coarse step
     h64 = {r.rid: r.history for r in seq64}

@@ -852,11 +852,12 @@ __device__ __forceinline__ void frontier_fluxes(const LevelView& L, int d, const
 // no element that is needed later depends on them.
 //   EDGE: the box reaches the ends of the array, where the stencils do not fit (faces 0,
 // 1 and the last along d, face 0 of the other axes).
-//   Bound by instruction issue (FP32 65-74 % of the issue slots, double-float 73-75 %).
-// Measured at a box of 136^3 (ncu, GB300): FP32 state x 33.0, y 32.1, z 32.4 us and 261 /
-// 276 / 266 thread instructions per cell, where an earlier form with blocks of 9 warps and
-// a barrier a plane took 363-400; double-float x 136, y 94, z 97 us and 1097 / 939 / 935
-// instructions.  Over a coarse step of 5 x 128^3 a sweep takes 40 us in FP32 and 122 in
+//   Bound by instruction issue (FP32 58-71 % of the issue slots, double-float 74-77 %).
+// Measured at the first sub-cycle of a 128^3 level (boxes of 136 x 140 x 140, 136 x 136 x
+// 140, 136^3; ncu, GB300): FP32 x 46.8, y 41.3, z 34.5 us and 288 / 319 / 326 thread
+// instructions per cell, where an earlier form with blocks of 9 warps and a barrier a plane
+// took 60-65 us at 144^3 and 363-400; double-float x 140, y 110, z 103 us and 1203 / 1117 /
+// 1128.  Over a coarse step of 5 x 128^3 a sweep takes 40 us in FP32 and 111 in
 // double-float, where that form took 68 us in FP32 and the four separate kernels 171 in
 // double-float.
 __device__ __forceinline__ float shfl_up(float v, int k) {
