@@ -456,6 +456,11 @@ struct LaunchDesc {
   unsigned nchunks;
 };
 
+// launches of a context whose items are passed by value
+bool by_value(const LaunchDesc& L) {
+  return L.nitems == 1 || (L.op == OP_COMMMEAN && L.d == kMeanWithFill);
+}
+
 struct Plan {
   int prec = 0;
   size_t item_size = 0;
@@ -938,6 +943,13 @@ struct Builder {
     add_force(r, true, out);
   }
 
+  // CommMean and the ghost fill that follows share a launch where they touch different
+  // levels: the next level step is then the parent's, or that of a level below the child
+  static bool mean_with_fill(const Entry& mean, const Entry& next) {
+    return mean.op == OP_COMMMEAN && next.op == OP_BC && mean.it.count && next.it.count &&
+           next.it.L.q[0] != mean.it.L.q[0] && next.it.L.q[0] != mean.it.F.q[0];
+  }
+
   // greedy merge: repeatedly launch the op kind that heads the most runs' lists,
   // taking it from every run whose next op it is (each run keeps its own order)
   void merge(Plan& plan) const {
@@ -983,6 +995,16 @@ struct Builder {
           }
           if (!is_joined_op(e.op)) break;
         }
+      }
+      if (!pool && pos[0] < per_run[0].size() && L.nitems == 1 &&
+          mean_with_fill(per_run[0][pos[0] - 1], per_run[0][pos[0]])) {
+        const Entry& e = per_run[0][pos[0]++];
+        const unsigned char* p = reinterpret_cast<const unsigned char*>(&e.it);
+        plan.items.insert(plan.items.end(), p, p + sizeof(Item<T>));
+        plan.starts.push_back(chunks);
+        chunks += (e.it.count + ce - 1) / ce;
+        L.nitems = 2;
+        L.d = kMeanWithFill;
       }
       L.nchunks = chunks;
       if (L.nitems) plan.launches.push_back(L);
@@ -1158,7 +1180,7 @@ long long plan_run(const Plan& plan, Exec& x, bool events) {
     unsigned grid = (unsigned)x.sm_count * (unsigned)x.bps[L.op];
     const Item<T>* it = (const Item<T>*)(items + L.item0 * plan.item_size);
     const unsigned* st = plan.d_starts + L.start0;
-    const Item<T>* hi = (L.nitems == 1 && x.single_fast)
+    const Item<T>* hi = (by_value(L) && x.single_fast)
                             ? (const Item<T>*)(plan.items.data() + L.item0 * plan.item_size)
                             : nullptr;
     if (events) {
@@ -1428,7 +1450,7 @@ int time_plan(const Plan& p, Exec& x, int prec, int bps, bool single_fast,
     for (size_t i = 0; i < p.launches.size(); ++i) {
       const LaunchDesc& L = p.launches[i];
       unsigned grid = (unsigned)x.sm_count * (unsigned)(bps > 0 ? bps : x.bps[L.op]);
-      const void* hi = (L.nitems == 1 && single_fast)
+      const void* hi = (by_value(L) && single_fast)
                            ? (const void*)(p.items.data() + L.item0 * p.item_size)
                            : nullptr;
       if (rep == 1) cudaEventRecord(ev[2 * i], x.st);

@@ -323,6 +323,9 @@ enum Op {
   OP_COUNT
 };
 
+// direction of an OP_COMMMEAN launch that holds a second item, an OP_BC of other levels
+constexpr int kMeanWithFill = 1;
+
 // ops whose consecutive items of one run are independent and share a launch
 __host__ __device__ constexpr bool is_joined_op(int op) {
   return op == OP_DT_LEVEL || op == OP_FORCE_LEVEL;
