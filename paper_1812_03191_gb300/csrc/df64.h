@@ -115,11 +115,13 @@ __host__ __device__ __forceinline__ df64 div_u(df64 a, df64 b) {
 }
 
 // A sum and a difference without the final renormalisation, for results that only feed
-// products, quotients and further sums: the value and its error are the operators', but
+// products, dividends and further sums: the value and its error are the operators', but
 // after a cancellation lo may be as large as hi.  It stays below 2^-23 (|a| + |b|), so
-// what a product or quotient drops of it (lo times the other operand's lo) is below
-// 2^-46 of |a| + |b| times that operand: the size of the sum's own error.  Not for sign
-// tests, canonical(), to_double() or an ordered comparison.
+// what a product drops of it (lo times the other operand's lo) is below 2^-46 of
+// |a| + |b| times that operand: the size of the sum's own error.  A divisor only where a
+// and b have the same sign: a quotient takes its reciprocal from hi and corrects once, so
+// it is off by (lo / hi)^2, the square of the cancellation.  Not for sign tests,
+// canonical(), to_double() or an ordered comparison.
 __host__ __device__ __forceinline__ df64 add_u(df64 a, df64 b) {
   const df64 s = two_sum(a.hi, b.hi);
   return df64(s.hi, s.lo + (a.lo + b.lo));
@@ -129,6 +131,10 @@ __host__ __device__ __forceinline__ df64 sub_u(df64 a, df64 b) { return add_u(a,
 __host__ __device__ __forceinline__ df64 fsub_u(float p, df64 a) {
   const df64 s = two_sum(p, -a.hi);
   return df64(s.hi, s.lo - a.lo);
+}
+// n / (a + b) for a sum that may cancel: normalised before it divides
+__host__ __device__ __forceinline__ df64 div_sum(df64 n, df64 a, df64 b) {
+  return div_u(n, a + b);
 }
 // any pair as a normalised one
 __host__ __device__ __forceinline__ df64 norm(df64 a) { return two_sum(a.hi, a.lo); }

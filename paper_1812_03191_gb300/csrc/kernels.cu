@@ -86,7 +86,9 @@ __device__ __forceinline__ df64 hdiv(df64 a, df64 b) { return a / b; }
 // without the final renormalisation (mul_u, div_u in df64.h), in FP32 the plain ones
 __device__ __forceinline__ float mul_u(float a, float b) { return a * b; }
 __device__ __forceinline__ float div_u(float a, float b) { return a * rcp_est(b); }
-// likewise the sum, the difference and p - a of a float p (add_u, sub_u, fsub_u there)
+// likewise the sum, the difference and p - a of a float p (add_u, sub_u, fsub_u there); a
+// sum that is divided by and may cancel (div_sum there)
+__device__ __forceinline__ float div_sum(float n, float a, float b) { return div_u(n, a + b); }
 __device__ __forceinline__ float add_u(float a, float b) { return a + b; }
 __device__ __forceinline__ float sub_u(float a, float b) { return a - b; }
 __device__ __forceinline__ float fsub_u(float p, float a) { return p - a; }
@@ -128,10 +130,13 @@ __device__ __forceinline__ df64 ky_add(df64 k, df64 y, df64 z) {
 }
 // e/rho - e0/rho0 of a cell from its deviations, (de - eps0 drho)/(rho0 + drho): one
 // expression for every kernel that forms it, so that all give the same bits.  Its
-// consumers only take differences of it, so the quotient stays unnormalised.
+// consumers only take differences of it, so the quotient stays unnormalised; dividend and
+// divisor are normalised, since both cancel where the gas is rarefied (left unnormalised,
+// the quotient was off by 6e-11 at a hundredth of the background density and by 6e-7 at
+// 1e-4, against 1.4e-12 and 1.5e-10, and a FP64 coarse step 0.9 % shorter).
 template <class C, class B>
 __device__ __forceinline__ C eps_dev(C de, C dr, const B& bg) {
-  return div_u(sub_u(de, mul_u(bg.eps0, dr)), add_u(bg.rho0, dr));
+  return div_sum(de - mul_u(bg.eps0, dr), bg.rho0, dr);
 }
 // a value as a store of the state keeps it (the FP64 state's stores cut lo)
 __device__ __forceinline__ float as_stored(float v) { return v; }
@@ -1029,8 +1034,8 @@ __device__ __forceinline__ void sweep_march(const Item<T>& it, int x, int row, b
     C w0[3];
 #pragma unroll
     for (int m = 0; m < 3; ++m) {
-      const C drf = halve(add_u(m == 0 ? rx : m == d ? r1 : rb, rc));
-      w0[m] = div_u(sub_ky(pc[m], bg.V[m], drf), add_u(bg.rho0, drf));
+      const C drf = halve((m == 0 ? rx : m == d ? r1 : rb) + rc);
+      w0[m] = div_sum(sub_ky(pc[m], bg.V[m], drf), bg.rho0, drf);
       if (EDGE && !(m == 0 ? x >= 1 : m == d ? r >= 1 && r < sM : row >= 1)) w0[m] = z;
     }
     const C dr0 = rc - r1, de0 = ep - e1, db0 = rb - b1;
