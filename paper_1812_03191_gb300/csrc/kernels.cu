@@ -1304,10 +1304,17 @@ __device__ __forceinline__ void sweep_x(const Item<T>& it, int x, int row, bool 
   }
 }
 
-// planes [m0, m1) of a column
-template <class T, int d>
+// planes [m0, m1) of a column.  BATCH, in a pool: every chunk of a box that reaches the ends
+// of the march takes the EDGE form, whose multiply-adds the compiler may contract otherwise,
+// so that a run's bits do not depend on where its pool's chunks end (FP32 runs with G = 2 or
+// 6 differed by roundings; 24 uneven FP32 runs a step, chosen by the chunk and by the box: with
+// viscosity 11.47 and 11.47 ms, with G = 6 6.91 and 6.91; chunks by the run alone instead 12.21
+// and 7.10).
+template <class T, int d, bool BATCH>
 __device__ __forceinline__ void sweep_column(const Item<T>& it, int col, int m0, int m1,
                                              Arith<T>* __restrict__ buf) {
+  constexpr int MU = d == 0 ? 2 : d;
+  const int e0 = BATCH ? it.b.lo[MU] : m0, e1 = BATCH ? it.b.hi[MU] : m1;
   constexpr int RA = d == 1 ? 2 : 1;
   const Box& b = it.b;
   SweepLane p;
@@ -1315,12 +1322,12 @@ __device__ __forceinline__ void sweep_column(const Item<T>& it, int col, int m0,
                   (int)(threadIdx.x & 31), p))
     return;
   if (d == 0) {
-    if (b.lo[0] >= 3 && b.hi[0] <= it.L.s[0] - 2 && b.lo[1] >= 1 && m0 >= 1)
+    if (b.lo[0] >= 3 && b.hi[0] <= it.L.s[0] - 2 && b.lo[1] >= 1 && e0 >= 1)
       sweep_x<T, false>(it, p.x, p.row, p.mine, m0, m1, buf);
     else
       sweep_x<T, true>(it, p.x, p.row, p.mine, m0, m1, buf);
   } else {
-    if (b.lo[0] >= 1 && b.lo[RA] >= 1 && m0 >= 3 && m1 <= it.L.s[d] - 2)
+    if (b.lo[0] >= 1 && b.lo[RA] >= 1 && e0 >= 3 && e1 <= it.L.s[d] - 2)
       sweep_march<T, d == 0 ? 1 : d, false>(it, p.x, p.row, p.mine && p.x >= b.lo[0], m0, m1, buf);
     else
       sweep_march<T, d == 0 ? 1 : d, true>(it, p.x, p.row, p.mine && p.x >= b.lo[0], m0, m1, buf);
@@ -1330,7 +1337,7 @@ __device__ __forceinline__ void sweep_column(const Item<T>& it, int col, int m0,
 // a unit of a sweep; ENDS: the columns are laid end to end (Box::zc < 0), a form of its own
 // because one form for both ran 0.6 % slower where chunks are taken (3 x 64^3 FP64 762 and
 // 766 us a coarse step)
-template <class T, int d, bool ENDS>
+template <class T, int d, bool ENDS, bool BATCH>
 __device__ __forceinline__ void el_sweep(const Item<T>& it, unsigned unit,
                                          Arith<T>* __restrict__ buf) {
   constexpr int MU = d == 0 ? 2 : d;
@@ -1342,13 +1349,13 @@ __device__ __forceinline__ void el_sweep(const Item<T>& it, unsigned unit,
     while (pos < end) {
       const int col = pos / nm, m0 = b.lo[MU] + pos - col * nm;
       const int m1 = min(m0 + end - pos, b.hi[MU]);
-      sweep_column<T, d>(it, col, m0, m1, buf);
+      sweep_column<T, d, BATCH>(it, col, m0, m1, buf);
       pos += m1 - m0;
     }
   } else {
     const int ncol = sweep_columns(b, d), chunk = (int)unit / ncol;
     const int m0 = b.lo[MU] + chunk * b.zc;
-    sweep_column<T, d>(it, (int)unit - chunk * ncol, m0, min(m0 + b.zc, b.hi[MU]), buf);
+    sweep_column<T, d, BATCH>(it, (int)unit - chunk * ncol, m0, min(m0 + b.zc, b.hi[MU]), buf);
   }
 }
 
@@ -2516,7 +2523,7 @@ __global__ void __launch_bounds__(kSweepThreads, sweep_blocks((int)sizeof(T), D)
   __shared__ Arith<T> s_planes[sweep_buffer((int)sizeof(T))];
   pdl_enter();
   if (skipped(it)) return;
-  el_sweep<T, D, ENDS>(it, blockIdx.x, s_planes + threadIdx.x);
+  el_sweep<T, D, ENDS, false>(it, blockIdx.x, s_planes + threadIdx.x);
   pdl_exit();
 }
 
@@ -2549,7 +2556,7 @@ __global__ void __launch_bounds__(kSweepThreads, sweep_blocks((int)sizeof(T), D)
       __syncthreads();
       cur = lo;
     }
-    if (!skipped(it)) el_sweep<T, D, false>(it, ch - starts[cur], s_planes + threadIdx.x);
+    if (!skipped(it)) el_sweep<T, D, false, true>(it, ch - starts[cur], s_planes + threadIdx.x);
     __syncthreads();
   }
   pdl_exit();
