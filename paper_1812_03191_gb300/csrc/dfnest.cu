@@ -12,6 +12,7 @@
 // the plan is uploaded once and captured into a CUDA graph, and the time step is
 // read by the kernels from device memory, so stepping never synchronises the host.
 // A context (df_ctx) is one run and its plan; a pool (df_pool) is many runs.
+#include <cuda.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -25,6 +26,7 @@
 #include <vector>
 
 #include "../../include/dfnest.h"
+#include "hostbuf.h"
 #include "internal.h"
 
 using namespace dfn;
@@ -1262,20 +1264,54 @@ double field_bg(const Run* r, int field) {
   return field == 0 ? r->P.rho0 : field == 1 ? r->P.e0 : r->P.V[field - 2];
 }
 
-// The device's address of a host buffer that it can reach by itself (pinned or registered
-// with CUDA, as its first and last value must be, 8-byte aligned), or null.
-double* mapped(const double* host, size_t n) {
-  if ((uintptr_t)host % sizeof(double)) return nullptr;
-  cudaPointerAttributes a{}, z{};
-  if (cudaPointerGetAttributes(&a, host) != cudaSuccess ||
-      cudaPointerGetAttributes(&z, host + n - 1) != cudaSuccess) {
+// the driver's answer about the range of an address; null where it has no such call
+using RangeFn = CUresult (*)(unsigned, CUpointer_attribute*, void**, CUdeviceptr);
+RangeFn range_fn() {
+  static const RangeFn fn = [] {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &f, 12000, cudaEnableDefault,
+                                         &q) != cudaSuccess ||
+        q != cudaDriverEntryPointSuccess) {
+      (void)cudaGetLastError();
+      return (RangeFn) nullptr;
+    }
+    return (RangeFn)f;
+  }();
+  return fn;
+}
+
+HostPart host_part(uintptr_t host, bool write) {
+  HostPart p = {};
+  cudaPointerAttributes a{};
+  if (cudaPointerGetAttributes(&a, (const void*)host) != cudaSuccess) {
     (void)cudaGetLastError();
-    return nullptr;
+    return p;
   }
-  if (a.type != cudaMemoryTypeHost || z.type != cudaMemoryTypeHost || !a.devicePointer ||
-      (const double*)z.devicePointer != (const double*)a.devicePointer + (n - 1))
-    return nullptr;
-  return (double*)a.devicePointer;
+  if (a.type != cudaMemoryTypeHost || !a.devicePointer || !range_fn()) return p;
+  CUdeviceptr start = 0;
+  CUpointer_attribute what[2] = {CU_POINTER_ATTRIBUTE_RANGE_START_ADDR,
+                                 CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+  void* to[2] = {&start, &p.size};
+  if (range_fn()(2, what, to, (CUdeviceptr)a.devicePointer) != CUDA_SUCCESS) return p;
+  p.pinned = true;
+  p.dev = (uintptr_t)a.devicePointer;
+  p.start = (uintptr_t)start;
+  unsigned flags = 0;
+  if (write && cudaHostGetFlags(&flags, (void*)host) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return p;
+  }
+  p.writable = write && !(flags & cudaHostRegisterReadOnly);
+  return p;
+}
+
+// The device's address of a host buffer that a kernel can read (`write`: write) by itself
+// (pinned or registered with CUDA from end to end, 8-byte aligned), or null.
+double* mapped(const double* host, size_t n, bool write) {
+  if ((uintptr_t)host % sizeof(double)) return nullptr;
+  return (double*)reachable((uintptr_t)host, n * sizeof(double), write,
+                            [&](uintptr_t at) { return host_part(at, write); });
 }
 
 // One field of one level to or from a host buffer; asynchronous where the buffer is
@@ -1289,7 +1325,7 @@ int run_io(Run* r, cudaStream_t st, int level, int field, double* out, const dou
   LevelView& v = r->L[level].v;
   size_t n = full ? (size_t)v.nc : (size_t)v.n[0] * v.n[1] * v.n[2];
   double bgv = raw ? 0.0 : field_bg(r, field);
-  double* direct = mapped(in ? in : out, n);
+  double* direct = mapped(in ? in : out, n, !in);
   if (in) {
     if (!direct)
       CK(cudaMemcpyAsync(r->stage, in, n * sizeof(double), cudaMemcpyHostToDevice, st));
