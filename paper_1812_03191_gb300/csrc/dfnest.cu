@@ -1344,13 +1344,23 @@ int io_async(Run* r, cudaStream_t st, int level, int field, double* out, const d
                             : run_io<float>(r, st, level, field, out, in, full, raw, launches);
 }
 
+// Waits for the transfers started on `st`; an error that is known already (`failed`) keeps
+// its message.
+int finish_transfers(cudaStream_t st, bool failed) {
+  const cudaError_t launched = failed ? cudaSuccess : cudaGetLastError();
+  const cudaError_t done = cudaStreamSynchronize(st);
+  if (failed) return DF_ECUDA;
+  CK(launched);
+  CK(done);
+  return DF_OK;
+}
+
 int io(Run* r, cudaStream_t st, int level, int field, double* out, const double* in, int full,
        bool raw, long long* launches) {
-  const int rc = io_async(r, st, level, field, out, in, full, raw, launches);
-  if (rc) return rc;
-  CK(cudaGetLastError());
-  CK(cudaStreamSynchronize(st));
-  return DF_OK;
+  return transfer_all(
+      1,
+      [&](int) { return io_async(r, st, level, field, out, in, full, raw, launches); },
+      [&](bool failed) { return finish_transfers(st, failed); });
 }
 
 }  // namespace
@@ -1831,14 +1841,13 @@ int df_get_state(df_ctx* c, double* out, double* t_out) {
   size_t nc = r->nc_max;
   DevGuard g(c->device);
   enter(c);
-  for (int l = 0; l < r->nl; ++l)
-    for (int f = 0; f < 5; ++f) {
-      int rc =
-          io_async(r, c->x.st, l, f, out + (l * 5 + f) * nc, nullptr, 1, true, &c->x.launches);
-      if (rc) return rc;
-    }
-  CK(cudaGetLastError());
-  CK(cudaStreamSynchronize(c->x.st));
+  const int rc = transfer_all(
+      5 * r->nl,
+      [&](int k) {
+        return io_async(r, c->x.st, k / 5, k % 5, out + k * nc, nullptr, 1, true, &c->x.launches);
+      },
+      [&](bool failed) { return finish_transfers(c->x.st, failed); });
+  if (rc) return rc;
   if (t_out) return df_status(c, t_out, nullptr, nullptr);
   return DF_OK;
 }
@@ -1850,16 +1859,19 @@ int df_set_state(df_ctx* c, const double* in, double t) {
   size_t nc = r->nc_max;
   DevGuard g(c->device);
   enter(c);
-  for (int l = 0; l < r->nl; ++l)
-    for (int f = 0; f < 5; ++f) {
-      int rc =
-          io_async(r, c->x.st, l, f, nullptr, in + (l * 5 + f) * nc, 1, true, &c->x.launches);
-      if (rc) return rc;
-    }
-  CK(cudaGetLastError());
-  CK(cudaMemcpyAsync(&r->ds->t, &t, sizeof(double), cudaMemcpyHostToDevice, c->x.st));
-  CK(cudaMemsetAsync(&r->ds->unhealthy, 0, sizeof(int), c->x.st));
-  CK(cudaStreamSynchronize(c->x.st));
+  const int n = 5 * r->nl;
+  const int rc = transfer_all(
+      n + 1,
+      [&](int k) -> int {
+        if (k < n)
+          return io_async(r, c->x.st, k / 5, k % 5, nullptr, in + k * nc, 1, true,
+                          &c->x.launches);
+        CK(cudaMemcpyAsync(&r->ds->t, &t, sizeof(double), cudaMemcpyHostToDevice, c->x.st));
+        CK(cudaMemsetAsync(&r->ds->unhealthy, 0, sizeof(int), c->x.st));
+        return DF_OK;
+      },
+      [&](bool failed) { return finish_transfers(c->x.st, failed); });
+  if (rc) return rc;
   r->stepped = false;
   return DF_OK;
 }
@@ -2226,14 +2238,24 @@ int df_pool_history(df_pool* p, int slot, int k, double* out, int* got) {
   CK(cudaStreamSynchronize(p->x.st));
   const long long m = std::min<long long>(std::min<long long>(k, pos), r->ring_cap);
   long long done = 0;
-  while (done < m) {  // at most two contiguous pieces of the ring
-    const long long e = pos - m + done, at = e % r->ring_cap;
-    const long long len = std::min(m - done, r->ring_cap - at);
-    CK(cudaMemcpyAsync(out + kRingStride * done, r->ring + kRingStride * at,
-                       kRingStride * len * sizeof(double), cudaMemcpyDeviceToHost, p->x.st));
-    done += len;
-  }
-  CK(cudaStreamSynchronize(p->x.st));
+  const int rc = transfer_all(
+      2,  // at most two contiguous pieces of the ring
+      [&](int) -> int {
+        const long long e = pos - m + done, at = e % r->ring_cap;
+        const long long len = std::min(m - done, r->ring_cap - at);
+        if (len > 0)
+          CK(cudaMemcpyAsync(out + kRingStride * done, r->ring + kRingStride * at,
+                             kRingStride * len * sizeof(double), cudaMemcpyDeviceToHost,
+                             p->x.st));
+        done += len;
+        return DF_OK;
+      },
+      [&](bool failed) -> int {
+        const cudaError_t e = cudaStreamSynchronize(p->x.st);
+        if (!failed) CK(e);
+        return DF_OK;
+      });
+  if (rc) return rc;
   *got = (int)m;
   return DF_OK;
 }

@@ -1,4 +1,5 @@
-// hostbuf.h -- which host buffers of the caller a kernel may read or write itself.
+// hostbuf.h -- which host buffers of the caller a kernel may read or write itself, and how
+// long.
 #pragma once
 
 #include <stddef.h>
@@ -33,6 +34,18 @@ uintptr_t reachable(uintptr_t host, size_t bytes, bool write, Ask ask) {
     done = rest < bytes - done ? done + rest : bytes;
   }
   return dev;
+}
+
+// Starts n transfers to or from the caller's buffer, up to the first that fails (issue(k)
+// gives a non-zero code), and then waits for those started in either case: when this returns
+// the device is done with the buffer.  The first code is returned; wait(failed) gives the
+// wait's own.
+template <class Issue, class Wait>
+int transfer_all(int n, Issue issue, Wait wait) {
+  int rc = 0;
+  for (int k = 0; k < n && !rc; ++k) rc = issue(k);
+  const int waited = wait(rc != 0);
+  return rc ? rc : waited;
 }
 
 }  // namespace dfn
