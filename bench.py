@@ -127,11 +127,12 @@ class ClockSampler:
 
 
 # --------------------------------------------------------------- algorithmic bytes
-# Arrays each stencil kernel reads + writes once per element of its box (the
-# compulsory traffic of the kernel as designed, neighbour reuse assumed cached).  The
-# boxes counted (level_step_boxes) are the active cells and the whole margin of the level
-# step; the library gives each operator only the margin that the next ones read, so these
-# bytes are an upper bound, 1.14 times the swept elements' for levels of 128^3.
+# Arrays each stencil kernel reads + writes once per element (the compulsory traffic of
+# the kernel as designed, neighbour reuse assumed cached).  The bandwidths that the lines
+# print count the active cells alone (bytes_per_launch with active=True): the boxes that the
+# operators run on hold a margin too, which depends on the operator and the level's size (the
+# swept elements of a finer level are 1.13 times the active cells at 128^3, 1.64 at 32^3),
+# so these bytes are a lower bound of what is moved.
 ARRAYS_PER_ELEM = {
     "source": 12,        # rho, e, phi, v3 -> v3, pi3
     "compress_lum": 8,   # e, v3, rho, lumw -> e, e/rho
@@ -145,6 +146,8 @@ ARRAYS_PER_ELEM = {
     "vrec_source": 9,    # rho, e, phi, pi3 -> v3
     "sweep": 11,         # fused sweep, the default: rho, e, pi3, v_d -> rho, e, pi3
 }
+# before fused sweeps the kick writes no momenta, and the x sweep reads rho, e, v3
+SWEPT_ARRAYS = {**ARRAYS_PER_ELEM, "source": 9, "sweep": 32 / 3}
 
 
 # DRAM bytes (read + write) of a launch per element of its level step's box, from the ncu
@@ -172,31 +175,50 @@ def level_step_boxes(cfg):
     return out
 
 
-def bytes_per_launch(cfg, kind, esz, fused=False):
+def bytes_per_launch(cfg, kind, esz, fused=False, active=False):
+    """Bytes of one launch of a kernel kind: over the mean box of level_step_boxes, or with
+    `active` over the active cells alone, with the arrays of the chosen transport."""
     boxes = level_step_boxes(cfg)
     n, G = cfg["n"], cfg["G"]
-    if kind in ARRAYS_PER_ELEM:
-        arrays = ARRAYS_PER_ELEM[kind] + (1 if kind == "diffuse" and not fused else 0)
-        return arrays * esz * sum(boxes) / len(boxes)
+    table = SWEPT_ARRAYS if fused and active else ARRAYS_PER_ELEM
+    if kind in table:
+        arrays = table[kind] + (1 if kind == "diffuse" and not fused else 0)
+        return arrays * esz * (n**3 if active else sum(boxes) / len(boxes))
     if kind == "commup":  # write every fine ghost element, read each coarse host once
-        return 5 * esz * (((n + 2 * G) ** 3 - n**3) + (n // 2 + G + 2) ** 3)
+        hosts = (n // 2 + G + 2) ** 3
+        if active:  # but not the hosts of the active cells, which no ghost reads
+            hosts -= (n // 2 - 2) ** 3
+        return 5 * esz * (((n + 2 * G) ** 3 - n**3) + hosts)
     if kind == "commmean":  # read 8 fine cells / 4 faces, write the covered coarse cell
+        if active:  # of the band along the child's frontier
+            band = cfg["params"]["band"]
+            cells = (n // 2) ** 3 - max(n // 2 - 2 * band, 0) ** 3
+            return (2 * 8 + 3 * 4 + 5) * esz * cells
         return 5 * esz * (n**3 + (n // 2) ** 3)
     return None
 
 
-def kernel_hbm_table(cfg, kinds, esz, fused, peak):
+def kernel_hbm_table(cfg, kinds, esz, fused, peak, active=False):
     """Algorithmic HBM bandwidth of every timed kernel kind with a byte count: bytes
-    per launch (ARRAYS_PER_ELEM over the mean box) / mean event-timed launch, and its
-    fraction of the peak."""
+    per launch (bytes_per_launch) / mean event-timed launch, and its fraction of the peak."""
     out = {}
     for kind, (ms, n) in kinds.items():
-        bpl = bytes_per_launch(cfg, kind, esz, fused)
+        bpl = bytes_per_launch(cfg, kind, esz, fused, active)
         if bpl is None or not n or ms <= 0:
             continue
         gbs = bpl / (ms / n / 1e3) / 1e9
         out[kind] = {"gbs": round(gbs, 1), "frac": round(gbs / peak, 3)}
     return out
+
+
+def pool_bytes_per_step(n, n_levels, kind, esz):
+    """Bytes of all launches of a stencil kind in one coarse step of one pool run, over the
+    active cells (the second sub-cycle of a finest level has no kick of its own)."""
+    steps = 2**n_levels - 1
+    if kind == "source" and n_levels > 1:
+        steps -= 2 ** (n_levels - 2)
+    launches = 3 * steps if kind == "sweep" else steps
+    return SWEPT_ARRAYS[kind] * esz * n**3 * launches
 
 
 def job_time_ms(ms, dist, device):
@@ -355,17 +377,10 @@ def run_batched(args):
     pool.set_timing(False)
     total_k = sum(v[0] for v in kinds.values())
     dom = max((k for k in kinds if k in ARRAYS_PER_ELEM), key=lambda k: kinds[k][0])
-    # algorithmic bytes of all launches of that kind in one step, from the runs' boxes
+    # algorithmic bytes of all launches of that kind in one step: the active cells of every
+    # level step (the pool's transport is the fused sweeps)
     esz = 4
-    per_step_bytes = 0.0
-    for r in runs:
-        swept = True  # the library's choice for the FP32 state in a pool of several runs
-        if (dom == "sweep" and not swept) or (dom in ("tprep", "tflux", "tmom", "tupdate")
-                                              and swept):
-            continue
-        boxes = level_step_boxes(dict(n=r["n"], G=r["G"], n_levels=r["n_levels"]))
-        mult = 3 if dom in ("tprep", "tflux", "tmom", "tupdate", "sweep") else 1
-        per_step_bytes += ARRAYS_PER_ELEM[dom] * esz * sum(boxes) * mult
+    per_step_bytes = sum(pool_bytes_per_step(r["n"], r["n_levels"], dom, esz) for r in runs)
     dom_ms, dom_n = kinds[dom]
     achieved = per_step_bytes * args.steps / (dom_ms / 1e3) / 1e9
     peak, peak_kind = peaks()
@@ -891,7 +906,8 @@ def main():
             "gpu_launches": m32["launches"], "clocks": m32["clocks"],
             "kernels_ms": {k: round(v[0], 4) for k, v in sorted(m32["kinds"].items(),
                                                                  key=lambda x: -x[1][0])},
-            "kernels_hbm": kernel_hbm_table(cfg, m32["kinds"], 4, fused32, peak),
+            "kernels_hbm": kernel_hbm_table(cfg, m32["kinds"], 4, fused32, peak,
+                                            active=True),
             "error_vs_fp64": {
                 "coarse_steps": args.warmup + 2 * args.steps,
                 "force_along_motion_rel": abs(F32 - F64) / abs(F64),
@@ -943,7 +959,7 @@ def main():
             "clocks": m["clocks"],
             "kernels_ms": {k: round(v[0], 4) for k, v in sorted(kinds.items(),
                                                                  key=lambda x: -x[1][0])},
-            "kernels_hbm": kernel_hbm_table(cfg, kinds, esz, fused, peak),
+            "kernels_hbm": kernel_hbm_table(cfg, kinds, esz, fused, peak, active=True),
             "force": {"F": list(m["F"]), "F_along_motion": m["Fmot"]},
         }
         if fp32 is not None:
