@@ -152,14 +152,15 @@ SWEPT_ARRAYS = {**ARRAYS_PER_ELEM, "source": 9, "sweep": 32 / 3}
 
 # DRAM bytes (read + write) of a launch per element of its level step's box, from the ncu
 # captures in profiles/ (k_sweep_fused_precision_5x128_fp32.md: fused sweeps of a 144^3 box,
-# 74.3 / 89.4 / 85.4 MB in FP32 and 223.7 / 224.3 / 202.4 MB in FP64; k_tmom_df64_nested_3x64.md:
-# double-float momentum fluxes of the separate transport kernels, 80^3 box, 20.09 / 20.09 /
-# 13.47 MB, a smaller case of the same kernel, whose traffic grows with the box); `traffic`
-# scales them to the mean box of the timed launches.  A kernel without a capture of its
-# current code reports null.
-_TMOM_DF64 = (20.0865e6 + 20.0840e6 + 13.4705e6) / 3 / 80**3
+# 74.3 / 89.4 / 85.4 MB in FP32 and 223.8 / 224.7 / 202.2 MB in FP64; k_tmom_df64_nested_3x64.md:
+# double-float momentum fluxes of the separate transport kernels, a smaller case of the same
+# kernel, whose traffic grows with the box: 20.08 / 20.09 MB on an 80^3 box and 13.47 on a
+# 72^3 one, all three counted per element of 80^3, so a tenth low); `traffic` scales them to
+# the mean box of the timed launches.  A kernel without a capture of its current code reports
+# null.
+_TMOM_DF64 = (20.0835e6 + 20.0852e6 + 13.4687e6) / 3 / 80**3
 TRAFFIC_PER_ELEM = {("precision_5x128^3", 4, "sweep"): (74.3e6 + 89.4e6 + 85.4e6) / 3 / 144**3,
-                    ("precision_5x128^3", 8, "sweep"): (223.7e6 + 224.3e6 + 202.4e6) / 3 / 144**3,
+                    ("precision_5x128^3", 8, "sweep"): (223.8e6 + 224.7e6 + 202.2e6) / 3 / 144**3,
                     ("precision_5x128^3", 8, "tmom"): _TMOM_DF64,
                     ("nested_3x64^3_fp64", 8, "tmom"): _TMOM_DF64}
 
@@ -734,7 +735,7 @@ B_ALG = {8: 80, 4: 40}
 # kernels launched once per level step (or per sweep of one), each over one level's
 # active cells: the units one launch processes are that level's cells
 LEVEL_STEP_KERNELS = ("source", "compress_lum", "diffuse", "tprep", "tflux", "tmom",
-                      "tupdate", "vrec_source", "sweep", "frontier_diff")
+                      "tupdate", "vrec_source", "sweep")
 
 
 def roofline_block(cfg, m, cu, esz, peak, peak_kind, fp64_peak=None):

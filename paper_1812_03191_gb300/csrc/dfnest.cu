@@ -504,17 +504,15 @@ int kind_of(int op) {
     case OP_SOURCE: return K_SOURCE;
     case OP_COMPRESS: return K_COMPRESS;
     case OP_DIFFUSE: return K_DIFFUSE;
-    case OP_FRONTIER_DIFF: return K_FRONTIER_DIFF;
     case OP_TPREP: return K_TPREP;
     case OP_TFLUX: return K_TFLUX;
-    case OP_TFRONTIER: return K_TFRONTIER;
     case OP_TMOM: return K_TMOM;
     case OP_TUPDATE: return K_TUPDATE;
     case OP_VREC: return K_VREC_SOURCE;
     case OP_COMMUP: return K_COMMUP;
     case OP_COMMMEAN: return K_COMMMEAN;
-    case OP_DT_LEVEL: case OP_DT_FINAL: return K_DT;
-    case OP_FORCE_LEVEL: case OP_FORCE_FINAL: return K_FORCE;
+    case OP_DT_LEVEL: return K_DT;
+    case OP_FORCE_LEVEL: return K_FORCE;
     case OP_SWEEP: return K_SWEEP;
     case OP_VISC_Q: case OP_VISC_V: return K_VISC;
     default: return K_OTHER;

@@ -314,8 +314,9 @@ struct DtFinal {
 // items; an item is one (run, level) with its box and its own parameters.
 // OP_TFRONTIER and OP_ZERO_ACC are no longer emitted (the CommFlux record replaced
 // them), nor are OP_DT_FINAL, OP_FORCE_FINAL and OP_TIME (the last chunk of OP_DT_LEVEL and
-// OP_FORCE_LEVEL does their work), nor OP_FRONTIER_DIFF (chunks of OP_DIFFUSE); they keep their numbers so that op indices (tile-shape
-// controls, timing kinds, the binding's op names) stay stable.
+// OP_FORCE_LEVEL does their work), nor OP_FRONTIER_DIFF (chunks of OP_DIFFUSE); they keep
+// their numbers so that op indices (tile-shape controls, the binding's op names) stay
+// stable, as K_FRONTIER_DIFF and K_TFRONTIER among the timing kinds do.
 enum Op {
   OP_SOURCE = 0, OP_COMPRESS, OP_FRONTIER_DIFF, OP_DIFFUSE, OP_TPREP, OP_TFLUX, OP_TFRONTIER,
   OP_TMOM, OP_TUPDATE, OP_VREC, OP_BC, OP_COMMUP, OP_COMMMEAN, OP_ZERO_ACC, OP_DT_LEVEL,

@@ -206,8 +206,9 @@ __device__ __forceinline__ C hslope(C dl, C dr) {
 // u <= 0 gives q0 + (-1 - cour)/2 * slope = q0 - (1 + cour)/2 * slope, with
 // (+-1 - cour)/2 * slope = (+-1 - cour) * hslope.  In double-float the operands of
 // the two one-sided differences are selected before subtracting (two subtractions of
-// 11 instructions, not three); in FP32 the three differences are formed and the
-// results selected, which measured faster in the fused sweeps (the same values).
+// 11 instructions, not three); in FP32, where a subtraction costs what a selection does,
+// the three differences are formed and the results selected (the same values).  The
+// separate transport kernels' form; the fused sweeps have the differences (upwind_d).
 template <class C>
 __device__ __forceinline__ C upwind_v(C qmm, C qm, C q0, C qp, C u, C cour) {
   const bool up = gt0(u);
@@ -841,9 +842,10 @@ __device__ __forceinline__ void frontier_fluxes(const LevelView& L, int d, const
 //   x sweep (sweep_x): the march is along z; the stencils' values come by warp shuffle, a
 // chunk starts one plane early (mass flux only).
 //   The rows are laid end to end, each with its halo (1 position below; x sweep: 3 below,
-// 2 above), and cut into warps that share 1 (5) positions, so that 96 % (81 %) of the
-// lanes own a cell whatever the box's width; a grid of 32-wide tiles left 80-85 %
-// (71-80 %).  The neighbour below in x comes by shuffle; of the row below the mass flux
+// 2 above), and cut into warps that share 1 (5) positions, so that 31/32 W/(W+1) of the
+// lanes own a cell of a box W wide (x sweep: 27/32 W/(W+5)): 96 % (81 %) at 136, 94 % (73 %)
+// at 32; a grid of 32-wide tiles left 80-85 % (71-80 %) at 136 to 144.  The neighbour below
+// in x comes by shuffle; of the row below the mass flux
 // is formed again from its rho and v_d (a tenth of the arithmetic), which costs less than
 // an exchange between warps: a tile in shared memory with three barriers a plane measured
 // 50 us against 37 at 136^3 (FP32, y), with the same arithmetic per cell.
@@ -857,12 +859,12 @@ __device__ __forceinline__ void frontier_fluxes(const LevelView& L, int d, const
 // no element that is needed later depends on them.
 //   EDGE: the box reaches the ends of the array, where the stencils do not fit (faces 0,
 // 1 and the last along d, face 0 of the other axes).
-//   Bound by instruction issue (FP32 58-71 % of the issue slots, double-float 74-77 %).
+//   Bound by instruction issue (FP32 58-71 % of the issue slots, double-float 75-77 %).
 // Measured at the first sub-cycle of a 128^3 level (boxes of 136 x 140 x 140, 136 x 136 x
 // 140, 136^3; ncu, GB300): FP32 x 46.8, y 41.3, z 34.5 us and 288 / 319 / 326 thread
 // instructions per cell, where an earlier form with blocks of 9 warps and a barrier a plane
-// took 60-65 us at 144^3 and 363-400; double-float x 140, y 110, z 103 us and 1203 / 1117 /
-// 1128.  Over a coarse step of 5 x 128^3 a sweep takes 40 us in FP32 and 111 in
+// took 60-65 us at 144^3 and 363-400; double-float x 143, y 111, z 105 us and 1211 / 1146 /
+// 1156.  Over a coarse step of 5 x 128^3 a sweep takes 40 us in FP32 and 113 in
 // double-float, where that form took 68 us in FP32 and the four separate kernels 171 in
 // double-float.
 __device__ __forceinline__ float shfl_up(float v, int k) {
@@ -927,7 +929,7 @@ struct Planes {
 //   Double-float: in shared memory, kSweepAhead planes ahead by asynchronous copies, each
 // thread's values in its own column of the buffer (so no barrier).  In registers they
 // would take 46: with the planes to come alone in shared memory the march needed 168 and
-// spilled, 138 us a sweep of 5 x 128^3 against 124 now with 152 (four blocks of 128
+// spilled, 138 us a sweep of 5 x 128^3 (in chunks) against 124 with 152 (four blocks of 128
 // registers spill again, 126).
 template <>
 struct Planes<df64> {
