@@ -511,8 +511,8 @@ int kind_of(int op) {
     case OP_VREC: return K_VREC_SOURCE;
     case OP_COMMUP: return K_COMMUP;
     case OP_COMMMEAN: return K_COMMMEAN;
-    case OP_DT_LEVEL: return K_DT;
-    case OP_FORCE_LEVEL: return K_FORCE;
+    case OP_DT_LEVEL: case OP_DT_FINAL: return K_DT;
+    case OP_FORCE_LEVEL: case OP_FORCE_FINAL: return K_FORCE;
     case OP_SWEEP: return K_SWEEP;
     case OP_VISC_Q: case OP_VISC_V: return K_VISC;
     default: return K_OTHER;
@@ -641,6 +641,19 @@ StepBoxes step_boxes(const Need& after, bool hydro, bool diffusion) {
   b.before.re = re;
   for (int d = 0; d < 3; ++d) b.before.v[d] = hydro ? v[d] : after.v[d];
   return b;
+}
+
+// Do the levels of a reduction share a launch, whose last chunk forms the result?  Always in a
+// pool; in a context up to so many chunks a level (time step: 1024 cells each, force: 2048):
+// each counts itself on one address, which costs large levels more (6 ns a chunk) than the
+// launches saved.  Joined and a launch a level, us per call of df_compute_dt (chunks a level):
+// FP64 3 x 64^3 (256) 47 and 48, 3 x 80^3 (500) 63 and 55, 3 x 112^3 (1372) 122 and 92, 2 x
+// 256^3 676 and 421, FP32 2 x 256^3 417 and 199; of df_force_now: FP64 3 x 64^3 (128) 46 and
+// 53, 3 x 96^3 (432) 83 and 75, 5 x 128^3 (1024) 245 and 205, FP32 220 and 223, 2 x 256^3
+// (8192) 625 and 568.  In a coarse step, whose launches follow each other at once, joined
+// gains up to about 900 chunks of the time step, 700 of the force, 1100 in FP32.
+constexpr bool joined_levels(int op, int esz, unsigned chunks, int levels) {
+  return chunks <= (op == OP_FORCE_LEVEL && esz == 4 ? 1500u : 700u) * (unsigned)levels;
 }
 
 template <class T>
@@ -906,25 +919,35 @@ struct Builder {
     return n;
   }
 
+  bool joined(const Run& r, int op) const {
+    return pool || joined_levels(op, (int)sizeof(T), chunks_of(r, op), r.nl);
+  }
+
   // the time step (Eq. 55) of a run
   void add_dt(const Run& r, int ri, std::vector<Entry>& out) const {
-    for (int l = 0; l < r.nl; ++l) {
-      Item<T> it = base(r, l);
+    const bool one = joined(r, OP_DT_LEVEL);
+    for (int l = 0; l <= r.nl; ++l) {
+      if (l == r.nl && one) break;
+      Item<T> it = base(r, l < r.nl ? l : 0);
       it.fin = d_fins + ri;
       it.n_levels = r.nl;
       it.total = chunks_of(r, OP_DT_LEVEL);
-      add(out, OP_DT_LEVEL, 0, it);
+      if (l < r.nl)
+        add(out, OP_DT_LEVEL, one ? 0 : kPerLevel, it);
+      else
+        add(out, OP_DT_FINAL, 0, it);
     }
   }
 
   // the force (Eq. 18) of a run; with `ring`, as the end of a coarse step: into the force
   // history, and the time advances
   void add_force(const Run& r, bool ring, std::vector<Entry>& out) const {
+    const bool one = joined(r, OP_FORCE_LEVEL);
     int off = 0;
-    for (int l = 0; l < r.nl; ++l) {
-      Item<T> it = base(r, l);
+    for (int l = 0; l <= r.nl; ++l) {
+      if (l == r.nl && one) break;
+      Item<T> it = base(r, l < r.nl ? l : 0);
       it.partials = r.partials + 3 * off;
-      off += force_partials_per_level(r.L[l].v);
       it.run_partials = r.partials;
       it.npart = r.n_partials;
       it.total = chunks_of(r, OP_FORCE_LEVEL);
@@ -933,7 +956,12 @@ struct Builder {
         it.ring_pos = r.ring_pos;
         it.ring_cap = r.ring_cap;
       }
-      add(out, OP_FORCE_LEVEL, 0, it);
+      if (l < r.nl) {
+        off += force_partials_per_level(r.L[l].v);
+        add(out, OP_FORCE_LEVEL, one ? 0 : kPerLevel, it);
+      } else {
+        add(out, OP_FORCE_FINAL, 0, it);
+      }
     }
   }
 
@@ -993,7 +1021,7 @@ struct Builder {
             chunks += nch;
             ++L.nitems;
           }
-          if (!is_joined_op(e.op)) break;
+          if (!is_joined_op(e.op, e.d)) break;
         }
       }
       if (!pool && pos[0] < per_run[0].size() && L.nitems == 1 &&

@@ -313,10 +313,10 @@ struct DtFinal {
 // Ops of the work-list kernel.  Every launch runs one op over a list of work
 // items; an item is one (run, level) with its box and its own parameters.
 // OP_TFRONTIER and OP_ZERO_ACC are no longer emitted (the CommFlux record replaced
-// them), nor are OP_DT_FINAL, OP_FORCE_FINAL and OP_TIME (the last chunk of OP_DT_LEVEL and
-// OP_FORCE_LEVEL does their work), nor OP_FRONTIER_DIFF (chunks of OP_DIFFUSE); they keep
-// their numbers so that op indices (tile-shape controls, the binding's op names) stay
-// stable, as K_FRONTIER_DIFF and K_TFRONTIER among the timing kinds do.
+// them), nor are OP_TIME (the force's end does its work) and OP_FRONTIER_DIFF (chunks of
+// OP_DIFFUSE); they keep their numbers so that op indices (tile-shape controls, the
+// binding's op names) stay stable, as K_FRONTIER_DIFF and K_TFRONTIER among the timing
+// kinds do.
 enum Op {
   OP_SOURCE = 0, OP_COMPRESS, OP_FRONTIER_DIFF, OP_DIFFUSE, OP_TPREP, OP_TFLUX, OP_TFRONTIER,
   OP_TMOM, OP_TUPDATE, OP_VREC, OP_BC, OP_COMMUP, OP_COMMMEAN, OP_ZERO_ACC, OP_DT_LEVEL,
@@ -327,9 +327,12 @@ enum Op {
 // direction of an OP_COMMMEAN launch that holds a second item, an OP_BC of other levels
 constexpr int kMeanWithFill = 1;
 
+// direction of a reduction whose levels have a launch each and whose end (OP_DT_FINAL,
+// OP_FORCE_FINAL) another
+constexpr int kPerLevel = 1;
 // ops whose consecutive items of one run are independent and share a launch
-__host__ __device__ constexpr bool is_joined_op(int op) {
-  return op == OP_DT_LEVEL || op == OP_FORCE_LEVEL;
+__host__ __device__ constexpr bool is_joined_op(int op, int d) {
+  return (op == OP_DT_LEVEL || op == OP_FORCE_LEVEL) && d != kPerLevel;
 }
 
 // ops that enumerate the elements of a box (the ones a tile shape applies to)

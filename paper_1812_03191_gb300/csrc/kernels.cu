@@ -1745,7 +1745,8 @@ __device__ __forceinline__ void el_commmean(const LevelView& C, const LevelView&
 // results are written; the last one clears the count for the next step.  Nothing waits.
 // The final step of a reduction then needs no launch of its own, and the levels share one
 // (one 32^3 level: 13 launches, 67.7 us a coarse step -> 10, 66.2; 3 x 64^3 FP64 69, 834
-// us -> 62, 800; 16 serving runs 99, 874 us -> 71, 770).
+// us -> 62, 800; 16 serving runs 99, 874 us -> 71, 770).  Large levels keep their launches
+// (joined_levels).
 __device__ __forceinline__ bool last_chunk(unsigned* done, unsigned total) {
   __shared__ int s_last;
   __syncthreads();
@@ -2412,12 +2413,16 @@ __device__ __forceinline__ void run_op(const Item<T>& it, unsigned tid) {
   else if (OP == OP_DT_LEVEL) {
     el_dt_level<T>(it.L, it.b, it.level, it.gg, it.gga, it.flags & FL_HYDRO, it.ds, it.rho0d, it.e0d,
                    it.V[0], it.V[1], it.V[2], it.bg, tid);
-    if (last_chunk(&it.ds->dt_done, it.total))
+    if (D != kPerLevel && last_chunk(&it.ds->dt_done, it.total))
       el_dt_finalize(it.ds, it.n_levels, *it.fin, it.dt_fixed);
   } else if (OP == OP_FORCE_LEVEL) {
     el_force_level<T>(it.L, it.b, it.L.fw, it.partials, tid);
-    if (last_chunk(&it.ds->force_done, it.total))
+    if (D != kPerLevel && last_chunk(&it.ds->force_done, it.total))
       el_force_finalize(it.run_partials, it.npart, it.ds, it.ring, it.ring_cap, it.ring_pos);
+  } else if (OP == OP_DT_FINAL) {
+    el_dt_finalize(it.ds, it.n_levels, *it.fin, it.dt_fixed);
+  } else if (OP == OP_FORCE_FINAL) {
+    el_force_finalize(it.run_partials, it.npart, it.ds, it.ring, it.ring_cap, it.ring_pos);
   }
 }
 
@@ -2602,7 +2607,7 @@ static void launch_one(const Item<T>* items, const unsigned* starts, int nitems,
                        unsigned grid, cudaStream_t st, const Item<T>* host_item) {
   if (nitems == 1 && host_item)
     launch_pdl(k_single<T, OP, D>, nchunks, kBlock, st, *host_item);
-  else if constexpr (is_joined_op(OP))
+  else if constexpr (is_joined_op(OP, D))
     launch_pdl(k_reduce<T, OP>, nchunks, kBlock, st, items, starts, nitems);
   else
     launch_pdl(k_batch<T, OP, D>, grid, kBlock, st, items, starts, nitems, nchunks);
@@ -2648,8 +2653,23 @@ int launch_batch(int op, int d, const Item<T>* items, const unsigned* starts, in
         launch_one<T, OP_COMMMEAN, 0>(items, starts, nitems, nchunks, grid, st, host_item);
       }
       break;
-    DFN_OP(OP_DT_LEVEL)
-    DFN_OP(OP_FORCE_LEVEL)
+    case OP_DT_LEVEL:  // d = kPerLevel: contexts only
+      if (d == 0) launch_one<T, OP_DT_LEVEL, 0>(items, starts, nitems, nchunks, grid, st, host_item);
+      else if (host_item)
+        launch_pdl(k_single<T, OP_DT_LEVEL, kPerLevel>, nchunks, kBlock, st, *host_item);
+      break;
+    case OP_FORCE_LEVEL:
+      if (d == 0)
+        launch_one<T, OP_FORCE_LEVEL, 0>(items, starts, nitems, nchunks, grid, st, host_item);
+      else if (host_item)
+        launch_pdl(k_single<T, OP_FORCE_LEVEL, kPerLevel>, nchunks, kBlock, st, *host_item);
+      break;
+    case OP_DT_FINAL:
+      if (host_item) launch_pdl(k_single<T, OP_DT_FINAL, 0>, nchunks, kBlock, st, *host_item);
+      break;
+    case OP_FORCE_FINAL:
+      if (host_item) launch_pdl(k_single<T, OP_FORCE_FINAL, 0>, nchunks, kBlock, st, *host_item);
+      break;
     DFN_OP(OP_VISC_Q)
     DFN_OP(OP_VISC_V)
     case OP_SWEEP:
