@@ -1257,12 +1257,23 @@ int plan_step(Plan& plan, Exec& x, int nsteps) {
   return DF_OK;
 }
 
+// What uploads to device memory that outlives the call, or waits, cannot be part of a capture
+// of the caller's stream, which `st` has joined: the upload would be recorded, not run.
+int check_not_capturing(cudaStream_t st) {
+  cudaStreamCaptureStatus s;
+  CK(cudaStreamIsCapturing(st, &s));
+  if (s == cudaStreamCaptureStatusNone) return DF_OK;
+  return fail(DF_ECUDA, "not possible while the stream is captured (a step is, once its plan is built)");
+}
+
 // run a list of ops of one run now, without a graph, and wait for it; `p` holds the
 // buffers, `ds` the scalars that a time step goes to; their copy to *out (nullable)
 int run_ops_now(Run* r, Exec& x, Plan& p, DevScalars* ds, DevScalars* out,
                 const std::vector<std::pair<int, int>>& ops) {
-  const int rc = r->prec == DF_FP64 ? plan_build_ops<double>(p, r, ds, x.st, ops)
-                                    : plan_build_ops<float>(p, r, ds, x.st, ops);
+  int rc = check_not_capturing(x.st);
+  if (!rc)
+    rc = r->prec == DF_FP64 ? plan_build_ops<double>(p, r, ds, x.st, ops)
+                            : plan_build_ops<float>(p, r, ds, x.st, ops);
   if (rc) return rc;
   x.launches += r->prec == DF_FP64 ? plan_run<double>(p, x, false) : plan_run<float>(p, x, false);
   cudaError_t e = cudaGetLastError();
@@ -1270,6 +1281,19 @@ int run_ops_now(Run* r, Exec& x, Plan& p, DevScalars* ds, DevScalars* out,
     e = cudaMemcpyAsync(out, ds, sizeof *out, cudaMemcpyDeviceToHost, x.st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(x.st);
   return e == cudaSuccess ? DF_OK : fail(DF_ECUDA, "ops: %s", cudaGetErrorString(e));
+}
+
+// scalars set to zero
+int new_scalars(const Allocator& al, cudaStream_t st, DevScalars** out) {
+  DevScalars* ds = nullptr;
+  CK(dev_alloc(al, (void**)&ds, sizeof *ds));
+  const cudaError_t e = cudaMemsetAsync(ds, 0, sizeof *ds, st);
+  if (e != cudaSuccess) {
+    dev_free(al, ds);
+    CK(e);
+  }
+  *out = ds;
+  return DF_OK;
 }
 
 struct DevGuard {
@@ -1449,6 +1473,8 @@ int sync_scalars(cudaStream_t st, Run* r, DevScalars* h) {
 
 int build_plan(Plan& p, const std::vector<Run*>& runs, int prec, int full_boxes,
                const TileTable& tiles, int transport, bool pool, const Exec& x) {
+  const int rc = check_not_capturing(x.st);
+  if (rc) return rc;
   return prec == DF_FP64
              ? plan_build<double>(p, runs, full_boxes, tiles, transport, pool, x.sm_count, x.st)
              : plan_build<float>(p, runs, full_boxes, tiles, transport, pool, x.sm_count, x.st);
@@ -1803,12 +1829,10 @@ int df_compute_dt(df_ctx* c, double* dt, double* dt_level) {
   enter(c);
   for (int l = 0; l < r->nl; ++l) r->xi[l] = 2;
   // into scalars of its own: the run's keep the last coarse step taken (df_status)
-  if (!c->dt_ds) {
-    CK(dev_alloc(r->al, (void**)&c->dt_ds, sizeof(DevScalars)));
-    CK(cudaMemsetAsync(c->dt_ds, 0, sizeof(DevScalars), c->x.st));
-  }
+  int rc = check_not_capturing(c->x.st);
+  if (!rc && !c->dt_ds) rc = new_scalars(r->al, c->x.st, &c->dt_ds);
   DevScalars after;
-  int rc = run_ops_now(r, c->x, c->ops, c->dt_ds, &after, {{OP_DT_LEVEL, 0}});
+  if (!rc) rc = run_ops_now(r, c->x, c->ops, c->dt_ds, &after, {{OP_DT_LEVEL, 0}});
   if (!rc && after.unhealthy) {
     CK(cudaMemcpyAsync(&r->ds->unhealthy, &after.unhealthy, sizeof(int), cudaMemcpyHostToDevice,
                        c->x.st));
