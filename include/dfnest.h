@@ -156,8 +156,7 @@ int df_set_params(df_ctx* ctx, const df_params* p);
  * t_out NULL: asynchronous on the context's stream, and DF_EUNHEALTHY is reported
  * by the next synchronising call.  t_out given: the call synchronises, writes the
  * simulated time after the steps and returns DF_EUNHEALTHY if the state went bad.
- * Within a capture of the caller's stream only with t_out NULL and after a step outside it
- * since the parameters were last set (DF_ECUDA otherwise). */
+ * Not within a capture of the caller's stream (DF_ECUDA). */
 int df_step(df_ctx* ctx, int n_coarse_steps, double* t_out);
 
 /* Synchronise, then return time, last coarse step and health (0 healthy). */

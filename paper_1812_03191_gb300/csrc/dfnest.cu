@@ -1263,7 +1263,7 @@ int check_not_capturing(cudaStream_t st) {
   cudaStreamCaptureStatus s;
   CK(cudaStreamIsCapturing(st, &s));
   if (s == cudaStreamCaptureStatusNone) return DF_OK;
-  return fail(DF_ECUDA, "not possible while the stream is captured (a step is, once its plan is built)");
+  return fail(DF_ECUDA, "not possible while the stream is being captured");
 }
 
 // run a list of ops of one run now, without a graph, and wait for it; `p` holds the
